@@ -782,7 +782,7 @@ tomo_status tomo_plan_create_ex(const tomo_geometry *g, const tomo_plan_options 
     if (ce == cudaSuccess)
       ce = cudaMemcpyAsync(tb + t_posd, H.pos_f.data(), sizeof(double) * H.pos_f.size(), cudaMemcpyHostToDevice, s);
     if (ce == cudaSuccess)
-      ce = launch_jacobi(p->d_inst, H.n, reinterpret_cast<double *>(tb + t_prof),
+      ce = launch_jacobi(p->d_inst, H.n_layers, H.J, H.n_max, reinterpret_cast<double *>(tb + t_prof),
                          reinterpret_cast<int *>(tb + t_poff), reinterpret_cast<double *>(tb + t_posd),
                          p->d_jdiag, I.jinv, H.precision, p->nc_max, -1.0, s);
     if (ce == cudaSuccess) {

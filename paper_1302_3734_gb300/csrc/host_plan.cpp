@@ -182,6 +182,7 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
     Nmin = std::min(Nmin, L.N);
     Nmax = std::max(Nmax, L.N);
   }
+  P->n_max = Nmax;
   // cluster size: every layer keeps >= 8 rows per CTA at level 1, unless the
   // caller asks for another power of two (1..16, at most N/2; streamed plans,
   // whose transforms use no cluster, up to 64 bands of the separate gather)

@@ -17,6 +17,7 @@ struct HostPlan {
   int n_layers = 0, n_wfs = 0, J = 0, Lf = 0, precond = 0, precision = 0;
   double alpha = 0.0, L0 = 0.0;
   int n = 0, n_slopes = 0, v_total = 0, C = 0;
+  int n_max = 0;                  // side of the largest layer
   int n_part = 0, cl_part_off = 0, upd_part_off = 0, fwd_part_off = 0, n_upd_blocks = 0;
   int n_lgs = 0;
   long long smem_transform = 0;   // dynamic shared memory of the synthesis kernel (bytes)

@@ -1201,87 +1201,189 @@ __global__ void __launch_bounds__(kThreads) k_slopes(const InstDev *__restrict__
 }
 
 // --------------------------------------------------------------- k_jacobi
-// Modified Jacobi diagonal (Sec. 5.1), exactly, at plan time:
+// Modified Jacobi diagonal (Sec. 5.1), exactly, at plan time and when alpha is retuned:
 //   J_lambda = sum_{m LGS} sigma_m^-2 ||Gamma_m P_m w_lambda||^2 + alpha D_lambda.
 // The basis function is separable, w = u(x) v(y), and so are the traced corner
 // coordinates, hence P_m w = U(a) V(b) and the Fried slopes are
 // sx = dU(a) mV(b), sy = mU(a) dV(b) (d: forward difference, m: two-point
-// mean).  Summing their squares over the valid subapertures of row b uses
-// prefix sums of dU^2 and mU^2 over the row's runs of valid subapertures.
-// One warp per coefficient; FP64 throughout.
-__global__ void k_jacobi(const InstDev *__restrict__ insts, const double *__restrict__ prof,
-                         const int *__restrict__ prof_off, const double *__restrict__ pos_fd,
-                         double *__restrict__ jdiag, void *jinv, int precision, int nc_max,
-                         double alpha) {
+// mean).  With Td(b), Tm(b) the sums of dU^2 and mU^2 over the valid
+// subapertures of row b, the norm is sum_b mV(b)^2 Td(b) + dV(b)^2 Tm(b).
+//
+// A CTA takes kJacTile columns (basis functions in x) and a group of rows
+// (basis functions in y) of one level's block, so that Td, Tm are formed once
+// per column and row of subapertures and V once per row, not once per
+// coefficient: prefix sums of dU^2, mU^2 per column (a warp scan), then in
+// chunks of 32 subaperture rows V^2 per row (lanes = b), Td, Tm per column
+// (lanes = columns, the row's runs of valid subapertures) and the products
+// (lanes = columns; only the rows b that a basis function reaches, a ballot
+// mask, since a Daubechies function has compact support).  FP64 throughout:
+// bound by the FP64 pipe, which issues one warp instruction in 16 cycles per
+// SM on this GPU.  Measured on GB300, E-ELT system: 377 us a call with its table
+// copies; one warp per coefficient with a serial prefix sum, dense over the
+// pupil, took 25.4 ms (and 5.4 s on the 100 m system).
+constexpr int kJacThreads = 256;
+constexpr int kJacRows = 32;    // rows (basis functions in y) per CTA at most
+constexpr int kJacChunk = 32;   // subaperture rows per pass
+
+// rows per CTA of a level block of side M: fewer for the coarse blocks, whose
+// functions span the whole pupil, so that their CTAs are no longer than the rest
+__host__ __device__ inline int jac_rows(int M) { return M >= 64 ? kJacRows : (M >= 32 ? 16 : 8); }
+
+// columns per CTA: 32, or fewer when the prefix sums of that many do not fit
+__host__ __device__ inline size_t jac_smem(int tw, int nc_max) {
+  const size_t stride = static_cast<size_t>((nc_max + 1) | 1);
+  return sizeof(double) * (2 * tw * stride + 2 * kJacChunk * tw + 2 * kJacRows * kJacChunk);
+}
+
+template <int TW>
+__global__ void __launch_bounds__(kJacThreads) k_jacobi(const InstDev *__restrict__ insts,
+                                                        const double *__restrict__ prof,
+                                                        const int *__restrict__ prof_off,
+                                                        const double *__restrict__ pos_fd,
+                                                        double *__restrict__ jdiag, void *jinv, int precision,
+                                                        int nc_max, double alpha) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned s_mask[kJacRows];
+  __shared__ unsigned s_need;
+  constexpr int RW = 32 / TW;                               // rows of one warp's lanes
+  constexpr int NA = kJacRows / (kJacThreads / 32) / RW;    // accumulators per lane
   const InstDev &I = insts[0];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int lam = blockIdx.x * (blockDim.x >> 5) + warp;
-  double *U = reinterpret_cast<double *>(smem_raw) + warp * 4 * (nc_max + 1);
-  double *V = U + (nc_max + 1);
-  double *Pd = V + (nc_max + 1);
-  double *Pm = Pd + (nc_max + 1);
-  if (lam >= I.n) return;
-  int l = 0;
-  while (l + 1 < I.n_layers && I.layers[l + 1].off <= lam) ++l;
+  const int J = I.J, k = J - static_cast<int>(blockIdx.y), l = blockIdx.z;   // coarse (longest) levels first
   const LayerDev &L = I.layers[l];
-  const int N = L.N, J = I.J;
-  const int rr = (lam - L.off) / N, cc = (lam - L.off) % N;
-  const int mx = rr > cc ? rr : cc;
-  int k = J;
-  for (int kk = 1; kk <= J; ++kk)
-    if (mx >= (N >> kk)) {
-      k = kk;
-      break;
-    }
-  const int H = (N >> (k - 1)) >> 1;
-  const int kx = cc < H ? 0 : 1, px = cc < H ? cc : cc - H;
-  const int ky = rr < H ? 0 : 1, py = rr < H ? rr : rr - H;
-  const double *ux = prof + prof_off[(l * (J + 1) + k) * 2 + kx];
-  const double *uy = prof + prof_off[(l * (J + 1) + k) * 2 + ky];
-  const int sx = px << k, sy = py << k;
-  double acc = 0.0;
+  const int N = L.N, M = N >> (k - 1), H = M >> 1, rows = jac_rows(M);
+  const int ntx = (M + TW - 1) / TW, nty = (M + rows - 1) / rows;
+  if (static_cast<int>(blockIdx.x) >= ntx * nty) return;
+  const int c0 = (static_cast<int>(blockIdx.x) % ntx) * TW, r0 = (static_cast<int>(blockIdx.x) / ntx) * rows;
+  if (k < J && c0 + TW <= H && r0 + rows <= H) return;      // all low-low: a coarser level's block
+  const int stride = (nc_max + 1) | 1;
+  double *Pd = reinterpret_cast<double *>(smem_raw);        // [TW][stride] prefix sums of dU^2
+  double *Pm = Pd + TW * stride;                            //   and of mU^2
+  double *Td = Pm + TW * stride;                            // [kJacChunk][TW]
+  double *Tm = Td + kJacChunk * TW;
+  double *Vm = Tm + kJacChunk * TW;                         // [kJacRows][kJacChunk] mV^2
+  double *Vd = Vm + kJacRows * kJacChunk;                   //   and dV^2
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kJacThreads / 32;
+  // first sample of basis function c of the block on the periodic grid, and its profile
+  auto shift = [&](int c) { return (c < H ? c : c - H) << k; };
+  auto profile = [&](int c) { return prof + prof_off[(l * (J + 1) + k) * 2 + (c < H ? 0 : 1)]; };
+  // samples of a level-k function that are not zero (0: the whole circle)
+  const long long sup = ((1LL << k) - 1) * (I.Lf - 1) + 1;
+  const int len = sup >= N ? N : static_cast<int>(sup);
+  // the function with profile u and shift s at traced corner (x0, f); false: zero there
+  auto reaches = [&](int x0, int s) { return ((x0 - s) & (N - 1)) < len || ((x0 + 1 - s) & (N - 1)) < len; };
+  auto value = [&](const double *u, int s, int x0, double f) {
+    return (1.0 - f) * u[(x0 - s) & (N - 1)] + f * u[(x0 + 1 - s) & (N - 1)];
+  };
+  double tot[NA];
+#pragma unroll
+  for (int i = 0; i < NA; ++i) tot[i] = 0.0;
   for (int m = 0; m < I.n_wfs; ++m) {
     const WfsDev &W = I.wfs[m];
     if (!W.is_lgs) continue;
     const int nc = W.nc, n = W.n;
     const int po = I.pos_off[m * I.n_layers + l];
-    for (int a = lane; a < nc; a += 32) {
-      const int x0 = I.pos_i0[po + a], y0 = I.pos_i0[po + nc + a];
-      const double fx = pos_fd[po + a], fy = pos_fd[po + nc + a];
-      U[a] = (1.0 - fx) * ux[(x0 - sx) & (N - 1)] + fx * ux[(x0 + 1 - sx) & (N - 1)];
-      V[a] = (1.0 - fy) * uy[(y0 - sy) & (N - 1)] + fy * uy[(y0 + 1 - sy) & (N - 1)];
-    }
-    __syncwarp();
-    if (lane == 0) {
-      Pd[0] = 0.0;
-      Pm[0] = 0.0;
-      for (int a = 0; a < n; ++a) {
-        const double d = U[a + 1] - U[a], mm = 0.5 * (U[a] + U[a + 1]);
-        Pd[a + 1] = Pd[a] + d * d;
-        Pm[a + 1] = Pm[a] + mm * mm;
+    const int *xi = I.pos_i0 + po, *yi = xi + nc;
+    const double *xf = pos_fd + po, *yf = xf + nc;
+    __syncthreads();   // the previous sensor's products are done with the prefix sums
+    for (int j = warp; j < TW; j += nw) {
+      const int c = c0 + j;
+      double cd = 0.0, cm = 0.0;   // sums before this chunk of 32 subapertures
+      if (lane == 0) Pd[j * stride] = Pm[j * stride] = 0.0;
+      const double *u = profile(c < M ? c : 0);
+      const int s = shift(c < M ? c : 0);
+      for (int a0 = 0; a0 < n; a0 += 32) {
+        const int a = a0 + lane;
+        const bool on = c < M && a < n && (reaches(xi[a], s) || reaches(xi[a + 1], s));
+        double d2 = cd, m2 = cm;
+        if (__any_sync(0xffffffffu, on)) {
+          d2 = m2 = 0.0;
+          if (on) {
+            const double u0 = value(u, s, xi[a], xf[a]), u1 = value(u, s, xi[a + 1], xf[a + 1]);
+            const double d = u1 - u0, mm = 0.5 * (u0 + u1);
+            d2 = d * d;
+            m2 = mm * mm;
+          }
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const double xd = __shfl_up_sync(0xffffffffu, d2, o), xm = __shfl_up_sync(0xffffffffu, m2, o);
+            if (lane >= o) {
+              d2 += xd;
+              m2 += xm;
+            }
+          }
+          d2 += cd;
+          m2 += cm;
+          cd = __shfl_sync(0xffffffffu, d2, 31);
+          cm = __shfl_sync(0xffffffffu, m2, 31);
+        }
+        if (a < n) {
+          Pd[j * stride + a + 1] = d2;
+          Pm[j * stride + a + 1] = m2;
+        }
       }
     }
-    __syncwarp();
-    double part = 0.0;
-    const int *rows = I.run_rows + W.run_off;
-    for (int b = lane; b < n; b += 32) {
-      const double dv = V[b + 1] - V[b], mv = 0.5 * (V[b] + V[b + 1]);
-      double sd = 0.0, sm = 0.0;
-      for (int q = rows[b]; q < rows[b + 1]; ++q) {
-        const int2 run = I.run_ab[q];
-        sd += Pd[run.y] - Pd[run.x];
-        sm += Pm[run.y] - Pm[run.x];
+    double part[NA];
+#pragma unroll
+    for (int i = 0; i < NA; ++i) part[i] = 0.0;
+    const int *runs = I.run_rows + W.run_off;
+    for (int b0 = 0; b0 < n; b0 += kJacChunk) {
+      if (threadIdx.x == 0) s_need = 0u;
+      __syncthreads();   // the prefix sums are written; the previous chunk's products are done
+      for (int i = warp; i < rows; i += nw) {
+        const int r = r0 + i, b = b0 + lane;
+        const int s = shift(r < M ? r : 0);
+        const bool on = r < M && b < n && (reaches(yi[b], s) || reaches(yi[b + 1], s));
+        const unsigned mask = __ballot_sync(0xffffffffu, on);
+        if (on) {
+          const double *u = profile(r);
+          const double v0 = value(u, s, yi[b], yf[b]), v1 = value(u, s, yi[b + 1], yf[b + 1]);
+          const double d = v1 - v0, mm = 0.5 * (v0 + v1);
+          Vd[i * kJacChunk + lane] = d * d;
+          Vm[i * kJacChunk + lane] = mm * mm;
+        }
+        if (lane == 0) {
+          s_mask[i] = mask;
+          if (mask) atomicOr(&s_need, mask);
+        }
       }
-      part += mv * mv * sd + dv * dv * sm;
+      __syncthreads();
+      const unsigned need = s_need;
+      for (int bl = warp; bl < kJacChunk; bl += nw) {
+        if (!((need >> bl) & 1u) || lane >= TW) continue;
+        double sd = 0.0, sm = 0.0;
+        for (int q = runs[b0 + bl]; q < runs[b0 + bl + 1]; ++q) {
+          const int2 run = I.run_ab[q];
+          sd += Pd[lane * stride + run.y] - Pd[lane * stride + run.x];
+          sm += Pm[lane * stride + run.y] - Pm[lane * stride + run.x];
+        }
+        Td[bl * TW + lane] = sd;
+        Tm[bl * TW + lane] = sm;
+      }
+      __syncthreads();
+      const int j = lane & (TW - 1), rl = lane / TW;
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        const int row = (warp + i * nw) * RW + rl;
+        unsigned mask = row < rows ? s_mask[row] : 0u;
+        while (mask) {
+          const int bl = __ffs(mask) - 1;
+          mask &= mask - 1u;
+          part[i] += Vm[row * kJacChunk + bl] * Td[bl * TW + j] + Vd[row * kJacChunk + bl] * Tm[bl * TW + j];
+        }
+      }
     }
-    acc += W.inv_sigma2 * part;
-    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < NA; ++i) tot[i] += W.inv_sigma2 * part[i];
   }
-  acc = warp_sum(acc);
-  if (lane == 0) {
-    // alpha < 0: the plan's own alpha D; otherwise alpha D for the given alpha
-    const double Jv = acc + (alpha < 0.0 ? L.dalpha[k] : alpha * L.dprior[k]);
+  // alpha < 0: the plan's own alpha D; otherwise alpha D for the given alpha
+  const double ad = alpha < 0.0 ? L.dalpha[k] : alpha * L.dprior[k];
+  const int cc = c0 + (lane & (TW - 1)), rl = lane / TW;
+#pragma unroll
+  for (int i = 0; i < NA; ++i) {
+    const int row = (warp + i * nw) * RW + rl, rr = r0 + row;
+    if (row >= rows || rr >= M || cc >= M || (k < J && rr < H && cc < H)) continue;
+    const int lam = L.off + rr * N + cc;
+    const double Jv = tot[i] + ad;
     jdiag[lam] = Jv;
     if (jinv) {
       if (precision) static_cast<double *>(jinv)[lam] = 1.0 / Jv;
@@ -1404,7 +1506,9 @@ cudaError_t configure_kernels() {
   if (e == cudaSuccess) e = configure_streamed_kernels();
   if (e == cudaSuccess) e = configure_gather_kernels();
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    e = cudaFuncSetAttribute(k_jacobi<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTransformSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_jacobi<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTransformSmem);
   return e;
 }
 
@@ -1468,16 +1572,22 @@ cudaError_t launch_slopes(int precision, const InstDev *insts, int n_wfs, int ma
   return cudaGetLastError();
 }
 
-cudaError_t launch_jacobi(const InstDev *insts, int n, const double *prof, const int *prof_off,
-                          const double *pos_fd, double *jdiag, void *jinv, int precision,
+cudaError_t launch_jacobi(const InstDev *insts, int n_layers, int J, int N_max, const double *prof,
+                          const int *prof_off, const double *pos_fd, double *jdiag, void *jinv, int precision,
                           int nc_max, double alpha, cudaStream_t s) {
-  const size_t per_warp = 4 * static_cast<size_t>(nc_max + 1) * sizeof(double);
-  int warps = static_cast<int>((96 * 1024) / per_warp);
-  warps = warps < 1 ? 1 : (warps > 8 ? 8 : warps);
-  const size_t smem = per_warp * warps;
-  const int blocks = (n + warps - 1) / warps;
-  k_jacobi<<<blocks, warps * 32, smem, s>>>(insts, prof, prof_off, pos_fd, jdiag, jinv, precision,
-                                           nc_max, alpha);
+  // 32 columns per CTA while their prefix sums fit (pupils up to about 360 subapertures), else 8
+  const int tw = jac_smem(32, nc_max) <= static_cast<size_t>(kMaxTransformSmem) ? 32 : 8;
+  const size_t smem = jac_smem(tw, nc_max);
+  int tiles = 1;
+  for (int k = 1; k <= J; ++k) {
+    const int M = N_max >> (k - 1), rows = jac_rows(M);
+    tiles = max(tiles, ((M + tw - 1) / tw) * ((M + rows - 1) / rows));
+  }
+  const dim3 g(tiles, J, n_layers);
+  if (tw == 32)
+    k_jacobi<32><<<g, kJacThreads, smem, s>>>(insts, prof, prof_off, pos_fd, jdiag, jinv, precision, nc_max, alpha);
+  else
+    k_jacobi<8><<<g, kJacThreads, smem, s>>>(insts, prof, prof_off, pos_fd, jdiag, jinv, precision, nc_max, alpha);
   return cudaGetLastError();
 }
 

@@ -66,10 +66,10 @@ cudaError_t launch_slopes(int precision, const InstDev *insts, int n_wfs, int ma
 
 // Exact modified Jacobi diagonal (single instance): diag(sum_LGS A~^T C~^-1 A~)
 // + alpha D into jdiag (alpha < 0: the plan's alpha), and its inverse into jinv
-// unless jinv is NULL.  prof,
+// unless jinv is NULL.  N_max: the largest layer's side; prof,
 // prof_off, pos_fd: the plan's basis profiles and FP64 corner fractions.
-cudaError_t launch_jacobi(const InstDev *insts, int n, const double *prof, const int *prof_off,
-                          const double *pos_fd, double *jdiag, void *jinv, int precision,
+cudaError_t launch_jacobi(const InstDev *insts, int n_layers, int J, int N_max, const double *prof,
+                          const int *prof_off, const double *pos_fd, double *jdiag, void *jinv, int precision,
                           int nc_max, double alpha, cudaStream_t s);
 
 }  // namespace tomo

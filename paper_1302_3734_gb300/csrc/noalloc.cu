@@ -78,7 +78,7 @@ extern "C" tomo_status tomo_jacobi_diagonal_noalloc(const tomo_plan *p, double a
     e = cudaMemcpyAsync(sb + b_prof + b_off, H.pos_f.data(), sizeof(double) * H.pos_f.size(),
                         cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
-    e = tomo::launch_jacobi(p->d_inst, H.n, reinterpret_cast<const double *>(sb),
+    e = tomo::launch_jacobi(p->d_inst, H.n_layers, H.J, H.n_max, reinterpret_cast<const double *>(sb),
                             reinterpret_cast<const int *>(sb + b_prof),
                             reinterpret_cast<const double *>(sb + b_prof + b_off), d_out, nullptr,
                             H.precision, p->nc_max, alpha, s);
