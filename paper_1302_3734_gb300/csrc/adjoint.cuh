@@ -161,6 +161,8 @@ struct TapRec {
   static constexpr int RS = KT <= 3 ? 4 : 8;   // T words per record
   int off;
   T w[KT];
+  // the first tap of a record alone
+  static __device__ __forceinline__ int offset(const T *rec) { return *reinterpret_cast<const int *>(rec); }
   __device__ __forceinline__ void load(const T *rec) {
     if constexpr (sizeof(T) == 4) {
       const float4 a = reinterpret_cast<const float4 *>(rec)[0];
@@ -202,13 +204,11 @@ __device__ __forceinline__ T window_sum(const T *__restrict__ p, int nc, const T
   return acc;
 }
 
-// Pupil-edge terms of the CTA's nodes: A[node] += sum over its entries of
-// (e_x t_x + e_y t_y) w (one short list per node, edge slots in s_coef).  The
-// entries of a node are read kEdgeBatch at a time (independent loads, which
-// matters when the lists are in global memory) and summed in list order.
+// Pupil-edge entries whose loads a thread issues together.
 constexpr int kEdgeBatch = 4;
 
-// The pupil-edge sum of one node over its entries [e0, e1), in list order.
+// The pupil-edge sum of one node over its entries [e0, e1), in list order: the
+// terms (e_x t_x + e_y t_y) w, edge slots in s_coef.
 template <typename T>
 __device__ __forceinline__ T edge_node_sum(int e0, int e1, const int *tk, const T *tw, const T *s_coef) {
   T acc = T(0);
@@ -227,12 +227,6 @@ __device__ __forceinline__ T edge_node_sum(int e0, int e1, const int *tk, const 
       if (b + u < e1) acc += s_coef[2 * k[u]] * wx[u] + s_coef[2 * k[u] + 1] * wy[u];
   }
   return acc;
-}
-
-template <typename T>
-__device__ __forceinline__ void gather_edges(int nn, const int *tn, const int *tb, const int *tk,
-                                             const T *tw, T *A, const T *s_coef) {
-  for (int j = threadIdx.x; j < nn; j += blockDim.x) A[tn[j]] += edge_node_sum<T>(tb[j], tb[j + 1], tk, tw, s_coef);
 }
 
 }  // namespace tomo

@@ -20,7 +20,7 @@ constexpr int kAnalysisThreads = 512;  // threads per CTA of the gather + analys
 constexpr int kAnalysisThreadsMax = 1024;  // ... when its shared memory leaves room for one
 constexpr int kSynthThreads = 512;     // threads per CTA of the synthesis kernel (at most)
 constexpr int kGatherThreads = 512;    // threads per CTA of the separate gather kernel
-constexpr int kMaxGatherSensors = 64;  // dense sensors the separate gather kernel stages
+constexpr int kMaxGatherSensors = 64;  // dense sensors the separate gather kernel lists
 constexpr int kUpdChunk = 1024;    // coefficients per pass of a vector-update CTA
 constexpr int kUpdMaxBlocks = 608; // update CTAs per instance at most (four per SM of 152 SMs)
 constexpr int kMaxTapsNode = 4;    // corners per axis whose bilinear taps reach one node
@@ -124,18 +124,18 @@ struct InstDev {
   const int *gt_ys;             // per row record: its window start in the staged v rows
   const int4 *vs_run;           // per (layer, rank, dense sensor): v run {g0, 16-byte words, smem offset}
   int vstage, v_total;          // staged v elements per analysis CTA; corner values of all sensors
-  int max_band_cells;           // separate gather: largest column sums of one (sensor, layer, band)
-  int max_band_v;               // ... and largest 16-byte-aligned run of its band rows of v (elements)
+  int max_band_v;               // separate gather: largest run of one band's corner rows of v (elements)
+  int gather_bands;             // bands per layer of gt_brows and tt_seg
   const int2 *gt_cols;          // per (m,l): columns [x, x+y) mod N_l that the sensor's taps reach
-  const int2 *gt_brows;         // per (m,l,rank): {v offset of the first corner row the band's row
-                                // records reach, number of rows}
+  const int4 *gt_brows;         // per (m,l,band): {v offset of the first corner row the band's row records
+                                // reach, number of rows; first node row with taps in the band, number}
   const void *stage_img;        // per (layer, rank): the CTA's stage image (img_stride bytes apart)
   long long img_stride;
   // Pupil-edge corrections: a tip/tilt-only sensor's corner field is
   // e_x t_x + e_y t_y and tip/tilt removal subtracts sigma^-2 (m_x t_x + m_y t_y),
   // with t = Gamma^T 1 nonzero on the pupil edge only; both reach the layers
   // through this sparse list.
-  const int2 *tt_seg;           // per (layer, cluster rank): [first, end) nodes with entries
+  const int2 *tt_seg;           // per (layer, band): [first, end) nodes with entries
   const int *tt_node;           // local node index (row-in-CTA * N + column)
   const int *tt_beg;            // entries [tt_beg[j], tt_beg[j+1]) of node j
   const int *tt_k;              // edge slot of the entry
@@ -244,27 +244,23 @@ TOMO_HD inline StageLayout stage_layout(int n_dense, int N, int R0, int rec_stri
 }
 
 // Shared-memory layout of the separate gather kernel (bytes, 16-byte aligned):
-// the band buffer of R0 x N nodes, the band's row records (first corner row,
-// KT weights per node row), the column-summed corner rows of one sensor (the
-// plan's largest band needs `cells` elements there), then, when the kernel
-// stages the corner rows it reads, `vcells` elements for one sensor's band
-// rows of v.
+// the band buffer of R0 x N nodes, then two stages of one sensor's band rows of
+// v, its N column records and R0 row records (offsets within a stage); at the end
+// the stages hold the band's pupil-edge terms (one element per entry).
 struct GatherSmem {
-  int ry, rw, u, v, total;
+  int stage, stage_bytes, xr, yr, total;
 };
-TOMO_HD inline GatherSmem gather_smem_layout(int R0, int N, int KT, int esz, long long cells, long long vcells,
-                                             bool vstage) {
+TOMO_HD inline GatherSmem gather_smem_layout(int R0, int N, int rec_stride, int esz, long long vcells) {
   GatherSmem g;
-  g.ry = (R0 * N * esz + 15) / 16 * 16;
-  g.rw = g.ry + (4 * R0 + 15) / 16 * 16;
-  g.u = g.rw + (R0 * KT * esz + 15) / 16 * 16;
-  g.v = g.u + static_cast<int>((cells * esz + 15) / 16 * 16);
-  g.total = g.v + (vstage ? static_cast<int>((vcells * esz + 15) / 16 * 16) : 0);
+  g.stage = R0 * N * esz;
+  g.xr = static_cast<int>((vcells * esz + 15) / 16 * 16);
+  g.yr = g.xr + N * rec_stride * esz;
+  g.stage_bytes = g.yr + R0 * rec_stride * esz;
+  g.total = g.stage + 2 * g.stage_bytes;
   return g;
 }
-// Shared memory up to which the gather kernel stages the corner rows (two CTAs
-// per SM keep fitting).
-constexpr int kGatherStageSmem = 104 * 1024;
+// Shared memory up to which a gather CTA takes a whole cluster band: two CTAs per SM.
+constexpr int kGatherSmem = 108 * 1024;
 
 // Work items.
 struct ClusterItem { int inst, layer; };

@@ -509,40 +509,11 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
       }
       P->gt_cols[m * P->n_layers + l] = cols;
     }
-  // per (sensor, layer, cluster rank): the corner rows that the row records of the
-  // rank's band of node rows reach, {v offset of the first row, row count}
-  P->gt_brows.assign(static_cast<size_t>(P->n_wfs) * P->n_layers * P->C, make_int2(0, 0));
-  P->max_band_cells = 0;
-  for (int m = 0; m < P->n_wfs; ++m)
-    for (int l = 0; l < P->n_layers; ++l) {
-      const int go = P->gt_off[m * P->n_layers + l];
-      if (go < 0) continue;
-      const WfsDev &d = P->wfs[m];
-      const int N = P->layers[l].N, R0 = N / P->C, KT = P->max_taps;
-      for (int c = 0; c < P->C; ++c) {
-        int lo = d.nc, hi = -1;
-        for (int k = c * R0; k < (c + 1) * R0; ++k) {
-          const int ro = P->gt_ro[go + N + k];
-          if (ro < 0) continue;
-          const int b0 = (ro - d.v_off) / d.nc;
-          lo = std::min(lo, b0);
-          hi = std::max(hi, std::min(d.nc, b0 + KT));
-        }
-        if (hi <= lo) continue;
-        P->gt_brows[(static_cast<size_t>(m) * P->n_layers + l) * P->C + c] = make_int2(d.v_off + lo * d.nc, hi - lo);
-        P->max_band_cells = std::max<long long>(P->max_band_cells,
-                                                static_cast<long long>(hi - lo) * P->gt_cols[m * P->n_layers + l].y);
-        // (KT more elements: a window's zero-weight taps may read past the rows when nc < KT)
-        const int vq = P->precision ? 2 : 4, start = d.v_off + lo * d.nc;
-        const long long run = start - start / vq * vq + static_cast<long long>(hi - lo) * d.nc + KT;
-        P->max_band_v = std::max<long long>(P->max_band_v, (run + vq - 1) / vq * vq);
-      }
-    }
   if (P->n_edge_wfs > 64) {
     *err = "more than 64 sensors with tip/tilt removal or tip/tilt-only measurement";
     return TOMO_ERR_UNSUPPORTED;
   }
-  // group the pupil-edge entries by (layer, cluster rank, node), and merge those
+  // sort the pupil-edge entries by (layer, node), and merge those
   // of one (node, edge slot): the slot's coefficients multiply the summed weights
   std::stable_sort(tt_entries.begin(), tt_entries.end(), [](const TTEntry &x, const TTEntry &y) {
     return x.layer != y.layer ? x.layer < y.layer : (x.node != y.node ? x.node < y.node : x.k < y.k);
@@ -560,12 +531,53 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
     }
     tt_entries.resize(w);
   }
-  P->tt_seg.assign(static_cast<size_t>(P->n_layers) * P->C, make_int2(0, 0));
-  {
+  // the tables of the gather over `bands` bands of rows per layer (a layer of fewer rows has
+  // one row per band)
+  auto build_bands = [&](int bands) {
+    // per (sensor, layer, band): the corner rows that the row records of the band's node rows
+    // reach, {v offset of the first row, row count}, and the node rows with taps, {first, count}
+    P->gather_bands = bands;
+    P->gt_brows.assign(static_cast<size_t>(P->n_wfs) * P->n_layers * bands, make_int4(0, 0, 0, 0));
+    P->max_band_cells = P->max_band_v = 0;
+    for (int m = 0; m < P->n_wfs; ++m)
+      for (int l = 0; l < P->n_layers; ++l) {
+        const int go = P->gt_off[m * P->n_layers + l];
+        if (go < 0) continue;
+        const WfsDev &d = P->wfs[m];
+        const int N = P->layers[l].N, nb = std::min(bands, N), R0 = N / nb, KT = P->max_taps;
+        for (int c = 0; c < nb; ++c) {
+          int lo = d.nc, hi = -1, k0 = -1, k1 = 0;
+          for (int k = c * R0; k < (c + 1) * R0; ++k) {
+            const int ro = P->gt_ro[go + N + k];
+            if (ro < 0) continue;
+            if (k0 < 0) k0 = k - c * R0;
+            k1 = k - c * R0 + 1;
+            const int b0 = (ro - d.v_off) / d.nc;
+            lo = std::min(lo, b0);
+            hi = std::max(hi, std::min(d.nc, b0 + KT));
+          }
+          if (hi <= lo) continue;
+          P->gt_brows[(static_cast<size_t>(m) * P->n_layers + l) * bands + c] =
+              make_int4(d.v_off + lo * d.nc, hi - lo, k0, k1 - k0);
+          P->max_band_cells = std::max<long long>(P->max_band_cells,
+                                                  static_cast<long long>(hi - lo) * P->gt_cols[m * P->n_layers + l].y);
+          // (KT more elements: a window's zero-weight taps may read past the rows when nc < KT; and
+          // the rows that a window of a sensor with nc < KT has below its field)
+          const int vq = P->precision ? 2 : 4, start = d.v_off + lo * d.nc;
+          const long long run = start % vq + static_cast<long long>(std::max(hi - lo, KT)) * d.nc + KT;
+          P->max_band_v = std::max<long long>(P->max_band_v, (run + vq - 1) / vq * vq);
+        }
+      }
+    // the pupil-edge entries by (layer, band, node)
+    P->tt_node.clear();
+    P->tt_beg.clear();
+    P->tt_k.clear();
+    P->tt_w.clear();
+    P->tt_seg.assign(static_cast<size_t>(P->n_layers) * bands, make_int2(0, 0));
     size_t e = 0;
     for (int l = 0; l < P->n_layers; ++l) {
-      const int N = P->layers[l].N, R0 = N / P->C;
-      for (int c = 0; c < P->C; ++c) {
+      const int N = P->layers[l].N, nb = std::min(bands, N), R0 = N / nb;
+      for (int c = 0; c < nb; ++c) {
         const int first = static_cast<int>(P->tt_node.size());
         while (e < tt_entries.size() && tt_entries[e].layer == l && tt_entries[e].node / N / R0 == c) {
           const int node = tt_entries[e].node;
@@ -578,31 +590,32 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
             ++e;
           }
         }
-        P->tt_seg[l * P->C + c] = make_int2(first, static_cast<int>(P->tt_node.size()));
+        P->tt_seg[static_cast<size_t>(l) * bands + c] = make_int2(first, static_cast<int>(P->tt_node.size()));
       }
     }
     P->tt_beg.push_back(static_cast<int>(P->tt_k.size()));
-  }
-  // the separate gather kernel's CTAs, one per (layer, band), costliest first so
-  // that the light bands fill the end of the launch; a band's cost counts its
-  // sensors' column sums and node rows, its pupil-edge entries and its grid rows
-  P->gather_items.clear();
-  for (int l = 0; l < P->n_layers; ++l) {
-    const int N = P->layers[l].N, R0 = N / P->C;
-    for (int c = 0; c < P->C; ++c) {
-      long long cost = static_cast<long long>(R0) * N / 4;
-      for (int m = 0; m < P->n_wfs; ++m) {
-        const int2 br = P->gt_brows[(static_cast<size_t>(m) * P->n_layers + l) * P->C + c];
-        const int ncol = P->gt_cols[m * P->n_layers + l].y;
-        if (br.y > 0 && ncol > 0) cost += static_cast<long long>(br.y + R0) * ncol;
+    // the separate gather kernel's CTAs, one per (layer, band), costliest first so
+    // that the light bands fill the end of the launch; a band's cost counts its
+    // sensors' column sums and node rows, its pupil-edge entries and its grid rows
+    P->gather_items.clear();
+    for (int l = 0; l < P->n_layers; ++l) {
+      const int N = P->layers[l].N, nb = std::min(bands, N), R0 = N / nb;
+      for (int c = 0; c < nb; ++c) {
+        long long cost = static_cast<long long>(R0) * N / 4;
+        for (int m = 0; m < P->n_wfs; ++m) {
+          const int4 br = P->gt_brows[(static_cast<size_t>(m) * P->n_layers + l) * bands + c];
+          const int ncol = P->gt_cols[m * P->n_layers + l].y;
+          if (br.y > 0 && ncol > 0) cost += static_cast<long long>(br.y + R0) * ncol;
+        }
+        const int2 seg = P->tt_seg[static_cast<size_t>(l) * bands + c];
+        cost += 4LL * (P->tt_beg[seg.y] - P->tt_beg[seg.x]);
+        P->gather_items.push_back({0, l, c, static_cast<int>(std::min<long long>(cost, INT_MAX))});
       }
-      const int2 seg = P->tt_seg[l * P->C + c];
-      cost += 4LL * (P->tt_beg[seg.y] - P->tt_beg[seg.x]);
-      P->gather_items.push_back({0, l, c, static_cast<int>(std::min<long long>(cost, INT_MAX))});
     }
-  }
-  std::stable_sort(P->gather_items.begin(), P->gather_items.end(),
-                   [](const PassItem &a, const PassItem &b) { return a.slot > b.slot; });
+    std::stable_sort(P->gather_items.begin(), P->gather_items.end(),
+                     [](const PassItem &a, const PassItem &b) { return a.slot > b.slot; });
+  };
+  build_bands(P->C);
   // staging of the gather tables in the analysis kernel, when it fits
   P->n_dense = 0;
   for (const auto &d : P->wfs) P->n_dense += d.kind != kTTOnly ? 1 : 0;
@@ -672,25 +685,39 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
     fits = fits && P->max_tt_entries <= 65535;   // the image's 16-bit entry indices
     P->gather_staged = fits ? 1 : 0;
     P->smem_analysis = fits ? need : P->smem_transform;
-    // the separate gather kernel: the band buffer (N/C rows of N), the band's row
-    // records, one sensor's column-summed corner rows, and the staged corner rows
-    // of two sensors where two CTAs per SM still fit
-    long long plain = 0, staged = 0;
+    // the separate gather kernel takes bands of this size at most: the band's nodes,
+    // its row records and the column sums of one sensor's corner rows within 220 KB
+    long long band = 0;
     for (const auto &d : P->layers) {
-      plain = std::max<long long>(plain, gather_smem_layout(d.N / P->C, d.N, P->max_taps, esz, P->max_band_cells,
-                                                            P->max_band_v, false).total);
-      staged = std::max<long long>(staged, gather_smem_layout(d.N / P->C, d.N, P->max_taps, esz, P->max_band_cells,
-                                                              P->max_band_v, true).total);
+      const long long R0 = d.N / P->C;
+      auto up = [](long long bytes) { return (bytes + 15) / 16 * 16; };
+      band = std::max(band, up(R0 * d.N * esz) + up(4 * R0) + up(R0 * P->max_taps * esz) + up(P->max_band_cells * esz));
     }
-    P->gather_vstage = staged <= kGatherStageSmem ? 1 : 0;
-    P->smem_gather = P->gather_vstage ? staged : plain;
-    if (!fits && P->smem_gather > 220LL * 1024) {
+    if (!fits && band > 220LL * 1024) {
       *err = "layer grids too large for the separate gather kernel's band buffers";
       return TOMO_ERR_UNSUPPORTED;
     }
     if (!fits && P->n_dense > kMaxGatherSensors) {
       *err = "more than 64 sensors with a dense corner field on layer grids too large for the staged gather";
       return TOMO_ERR_UNSUPPORTED;
+    }
+    // the separate gather's bands: the cluster bands, halved until a CTA's buffers leave room for
+    // two CTAs per SM (at the latest at one node row per band)
+    auto smem_bands = [&]() {
+      int entries = 0;
+      for (const auto &sg : P->tt_seg) entries = std::max(entries, P->tt_beg[sg.y] - P->tt_beg[sg.x]);
+      int most = 0;
+      for (const auto &d : P->layers) {
+        const GatherSmem g = gather_smem_layout(d.N / std::min(P->gather_bands, d.N), d.N, P->rec_stride, esz,
+                                                P->max_band_v);
+        most = std::max(most, std::max(g.total, g.stage + entries * esz));
+      }
+      return most;
+    };
+    P->smem_gather = smem_bands();
+    while (!fits && P->smem_gather > kGatherSmem && P->gather_bands < Nmax) {
+      build_bands(2 * P->gather_bands);
+      P->smem_gather = smem_bands();
     }
   }
   // the stage images, one per analysis CTA

@@ -61,6 +61,8 @@ __device__ __forceinline__ void bulk_copy_g2s(void *dst, const void *src, uint32
 }
 // global data that an earlier grid wrote, about to be read by bulk copies
 __device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;\n" ::: "memory"); }
+// shared memory that this thread wrote, before a later bulk copy into it
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
   for (int i = 0; i < kMbarSpins; ++i) {
     uint32_t done;
