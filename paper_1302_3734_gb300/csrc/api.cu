@@ -540,7 +540,7 @@ tomo_status tomo_plan_create_ex(const tomo_geometry *g, const tomo_plan_options 
   }
   const size_t esz = H.precision ? 8 : 4;
   p->esz = esz;
-  if (forward_smem(H.n_layers, H.precision) > static_cast<size_t>(kMaxForwardSmem)) {
+  if (H.n_layers > kMaxForwardLayers[H.precision]) {
     delete p;
     return fail(TOMO_ERR_UNSUPPORTED, "too many layers for the forward kernel's staged tables");
   }

@@ -11,11 +11,13 @@ namespace tomo {
 
 constexpr int kMaxTaps = 8;        // Daubechies order <= 4
 constexpr int kMaxLevels = 12;
-constexpr int kFwdTile = 16;       // corners per side of a forward tile
+constexpr int kFwdTile = 16;       // subapertures per side of a mirror-slope tile
+constexpr int kFwdCols = 30, kFwdRows = 14;   // corners of a forward tile (with its halo 32 x 16)
+constexpr int kFwdThreads = 128;   // threads of a forward CTA in big launches (four times that in small ones)
+constexpr int kFwdChunk = 512;     // (edge corner, layer) pairs of a tip/tilt-only forward CTA
 constexpr int kMaxBatch = 96;      // instances per launch (kernel-argument arrays)
 constexpr int kThreads = 256;      // threads per CTA of the hot kernels (transforms: below)
-constexpr int kFwdThreads = 512;   // largest forward CTA; small launches use it, big batches kThreads
-constexpr int kFwdSmallLaunch = 608;   // forward CTAs up to which a launch uses kFwdThreads
+constexpr int kFwdSmallLaunch = 608;   // forward CTAs up to which a launch is small
 constexpr int kAnalysisThreads = 512;  // threads per CTA of the gather + analysis kernel when two fit an SM
 constexpr int kAnalysisThreadsMax = 1024;  // ... when its shared memory leaves room for one
 constexpr int kSynthThreads = 512;     // threads per CTA of the synthesis kernel (at most)
@@ -288,7 +290,8 @@ TOMO_HD inline int pass_smem_elems(int M, int LF) {
   const int s = 4 * (kPassRows + LF / 2 - 1) * M;
   return a > s ? a : s;
 }
-struct FwdItem { int inst, wfs, a0, b0, tile, pad0, pad1, pad2; };  // a0 < 0: tip/tilt-only sensor
+// A tile of a sensor (a0 < 0: a chunk of a tip/tilt-only sensor); pos: the sensor's corner tables.
+struct FwdItem { int inst, wfs, a0, b0, tile, pos, pad1, pad2; };
 struct UpdItem { int inst, start, blk, chunks; };   // chunks: passes of kUpdChunk coefficients
 
 }  // namespace tomo

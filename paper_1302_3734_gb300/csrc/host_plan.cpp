@@ -836,26 +836,26 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
   P->fwd_part_off = part;
   for (int m = 0; m < P->n_wfs; ++m) {
     WfsDev &d = P->wfs[m];
+    const int pos = P->pos_off[m * P->n_layers];   // the layers' tables follow each other, 2 nc entries each
     d.part_off = part;
     if (d.kind == kTTOnly) {
       // (edge corner, layer) pairs, one per thread of a chunk
       const int pairs = d.n_edge * P->n_layers;
-      const int chunks = (pairs + kThreads - 1) / kThreads;
+      const int chunks = (pairs + kFwdChunk - 1) / kFwdChunk;
       d.n_tiles = chunks;
-      for (int c = 0; c < chunks; ++c) P->fwd_items.push_back({0, m, -1, 0, c, 0, 0, 0});
+      for (int c = 0; c < chunks; ++c) P->fwd_items.push_back({0, m, -1, 0, c, pos, 0, 0});
       part += 2 * chunks;
       continue;
     }
-    const int nt = (d.nc + kFwdTile - 1) / kFwdTile;
     int tiles = 0;
-    for (int tb = 0; tb < nt; ++tb)
-      for (int ta = 0; ta < nt; ++ta) {
+    for (int b0 = 0; b0 < d.nc; b0 += kFwdRows)
+      for (int a0 = 0; a0 < d.nc; a0 += kFwdCols) {
         bool any = false;
-        for (int b = tb * kFwdTile; b < std::min(d.nc, (tb + 1) * kFwdTile) && !any; ++b)
-          for (int a = ta * kFwdTile; a < std::min(d.nc, (ta + 1) * kFwdTile) && !any; ++a)
+        for (int b = b0; b < std::min(d.nc, b0 + kFwdRows) && !any; ++b)
+          for (int a = a0; a < std::min(d.nc, a0 + kFwdCols) && !any; ++a)
             any = P->active[d.act_off + b * d.nc + a] != 0;
         if (!any) continue;
-        P->fwd_items.push_back({0, m, ta * kFwdTile, tb * kFwdTile, tiles, 0, 0, 0});
+        P->fwd_items.push_back({0, m, a0, b0, tiles, pos, 0, 0});
         ++tiles;
       }
     d.n_tiles = tiles;

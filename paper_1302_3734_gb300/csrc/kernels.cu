@@ -94,142 +94,234 @@ __device__ __forceinline__ T trace_corner(const InstDev &I, int m, int nc, const
 // io.in0: layer grids (NULL = the plan's phi); io.in1: slopes (MODE 1, 2).
 // EL: some sensor of the launch has elongated spots (Sec. 4.3); without it the
 // elongation code is compiled out.
-// Launched with kThreads or kFwdThreads threads.  The per-corner steps use
-// every thread; the steps that feed the tile's partial sums (the slopes and
-// the tip/tilt-only chunks) keep a fixed kThreads-thread mapping, so the
-// partials, and every result, are bitwise the same at either block size.
-constexpr int kHalo = kFwdTile + 2;
+//
+// A tile is kFwdCols x kFwdRows corners of a sensor.  The ray-trace covers the
+// tile and a halo of one corner, kFwdLanes columns (one per lane) by kFwdPsi
+// rows, RS consecutive rows per warp.  Down a column the corners' traced rows
+// follow each other on the layer grid, mostly one node row apart or, under the
+// cone effect, in the same one, so the interpolation along x of a node row is
+// formed once for the corner rows above and below it: RS + 1 node rows are read
+// per layer instead of 2 RS, all requested before any is used.
+//
+// RS = 4 (kFwdThreads threads) for big launches, RS = 1 (four times the
+// warps, no reuse, less work in a chain) for small ones.  The steps that feed
+// the tile's partial sums (the slopes and the tip/tilt-only chunks) keep a
+// fixed kFwdThreads-thread mapping, so the partials, and every result, are
+// bitwise the same at either block size.
+//
+// Bound by instruction issue and L1 in big launches, by latency in small ones.
+// Against one corner per thread on 18 x 18 corners, four loads per corner and
+// layer (GB300, cold launch): 16 E-ELT systems 49.2 -> 33 us, 64 uneven systems
+// 50.9 -> 34 us, the 100 m system 54.0 -> 46 us.
+constexpr size_t kFwdSmallSmem = 64 * 1024;
+constexpr int kFwdLanes = kFwdCols + 2, kFwdPsi = kFwdRows + 2;
 
-__host__ __device__ constexpr size_t fwd_table_bytes(int L, size_t esz) {
-  return ((sizeof(int) * (2 * L + 2 * L * kHalo) + 15) & ~size_t(15)) + 2 * L * kHalo * esz;
+// Shared memory of the staged corner tables of L layers: per layer the grid
+// side and offset, the columns' node index and fraction, and per corner row
+// (first node row * N, fraction).
+template <typename T>
+struct FwdRow {
+  int r0;
+  T f;
+};
+template <typename T>
+__host__ __device__ constexpr size_t fwd_table_bytes(int L) {
+  return L * (kFwdPsi * sizeof(FwdRow<T>) + kFwdLanes * sizeof(T) + (kFwdLanes + 2) * sizeof(int)) + 16;
 }
 
-// NT: the block size the instance is compiled for: kFwdThreads with two CTAs
-// per SM for small launches, kThreads with kFwdBatchBlocks CTAs per SM (fewer
-// registers) for big ones (FP32; FP64 instances keep the registers they need).
-constexpr int kFwdBatchBlocks = 5;
+// (1 - f) a + f b, rounded the same way wherever it is used.
+__device__ __forceinline__ float lerp(float f, float a, float b) {
+  return __fmaf_rn(__fsub_rn(1.f, f), a, __fmul_rn(f, b));
+}
+__device__ __forceinline__ double lerp(double f, double a, double b) {
+  return __fma_rn(__dsub_rn(1.0, f), a, __dmul_rn(f, b));
+}
 
-template <typename T, int MODE, bool EL, int NT>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT == kFwdThreads ? 2 : kFwdBatchBlocks) : 1)
+// The corners' phase psi = sum_l phi_l(traced corner) for RS rows from corner
+// row w of the tile's psi rows, lane = column; layers in order.
+template <typename T, int RS>
+__device__ __forceinline__ void trace_strip(const T *__restrict__ phi, int L, int w, const int *s_N, const int *s_off,
+                                            const int *s_x0, const T *s_fx, const FwdRow<T> *s_row, T (&val)[RS]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int j = 0; j < RS; ++j) val[j] = T(0);
+  // layers whose loads are in flight together
+  constexpr int kBatch = RS == 1 ? 4 : 2;
+  for (int l0 = 0; l0 < L; l0 += kBatch) {
+    T v0[kBatch][RS + 1], v1[kBatch][RS + 1], fx[kBatch], fy[kBatch][RS];
+    int r0[kBatch][RS], mask[kBatch];
+    bool odd = false;
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int l = l0 + q < L ? l0 + q : L - 1;
+      const int N = s_N[l], x0 = s_x0[l * kFwdLanes + lane];
+      fx[q] = s_fx[l * kFwdLanes + lane];
+      mask[q] = N * N - 1;
+      const T *p0 = phi + s_off[l] + x0, *p1 = phi + s_off[l] + ((x0 + 1) & (N - 1));
+      int last = 0;
+#pragma unroll
+      for (int j = 0; j < RS; ++j) {
+        const FwdRow<T> row = s_row[l * kFwdPsi + w + j];
+        const int r1 = (row.r0 + N) & mask[q];
+        r0[q][j] = row.r0;
+        fy[q][j] = row.f;
+        if (j == 0) {
+          v0[q][0] = p0[row.r0];
+          v1[q][0] = p1[row.r0];
+        } else {
+          odd = odd || (row.r0 != last && row.r0 != r0[q][j - 1]);
+        }
+        v0[q][j + 1] = p0[r1];
+        v1[q][j + 1] = p1[r1];
+        last = r1;
+      }
+    }
+    const bool skips = RS > 1 && __any_sync(0xffffffffu, odd);   // (the same in every lane)
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      if (l0 + q >= L) break;
+      T h0 = lerp(fx[q], v0[q][0], v1[q][0]);
+      T h1 = lerp(fx[q], v0[q][1], v1[q][1]);
+#pragma unroll
+      for (int j = 0; j < RS; ++j) {
+        if (j > 0) {
+          if (skips) {
+            // a node row between is skipped somewhere (subapertures larger than the layer's cells)
+            const int l = l0 + q, N = s_N[l], x0 = s_x0[l * kFwdLanes + lane];
+            const T *p = phi + s_off[l] + r0[q][j];
+            h0 = lerp(fx[q], p[x0], p[(x0 + 1) & (N - 1)]);
+          } else {
+            h0 = r0[q][j] == r0[q][j - 1] ? h0 : h1;
+          }
+          h1 = lerp(fx[q], v0[q][j + 1], v1[q][j + 1]);
+        }
+        val[j] += lerp(fy[q][j], h0, h1);
+      }
+    }
+  }
+}
+
+template <typename T, int MODE, bool EL, int RS>
+__global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
     k_forward(const InstDev *__restrict__ insts, const FwdItem *__restrict__ items, IoArgs io) {
   extern __shared__ __align__(16) unsigned char fsm[];
-  __shared__ InstDev sI;
-  __shared__ T s_psi[kHalo][kHalo + 1];
-  __shared__ T s_ex[kFwdTile + 1][kFwdTile + 2];
-  __shared__ T s_ey[kFwdTile + 1][kFwdTile + 2];
+  __shared__ T s_psi[kFwdPsi][kFwdLanes + 1];
+  __shared__ T s_ex[kFwdRows + 1][kFwdLanes];
+  __shared__ T s_ey[kFwdRows + 1][kFwdLanes];
   pdl_trigger();
   const FwdItem it = items[blockIdx.x];
   if (io.active && !io.active[it.inst]) return;
-  load_inst(&sI, insts + it.inst);
-  const InstDev &I = sI;
-  const WfsDev W = I.wfs[it.wfs];
+  const InstDev &I = insts[it.inst];
+  const WfsDev W = I.wfs[it.wfs];   // (by value: nothing of it is read again after the dependency wait)
   const T *phi = io.in0[it.inst] ? static_cast<const T *>(io.in0[it.inst]) : static_cast<const T *>(I.phi);
   const T *dat = static_cast<const T *>(io.in1[it.inst]);
-  const int nc = W.nc, n = W.n, tid = threadIdx.x, L = I.n_layers;
+  const int nc = W.nc, n = W.n, tid = threadIdx.x, nt = blockDim.x, L = I.n_layers;
+  const int *pi = I.pos_i0 + it.pos;   // the sensor's corner tables: per layer nc columns, then nc rows
+  const T *pf = static_cast<const T *>(I.pos_f) + it.pos;
+  double *part = I.part + W.part_off;
+  T *v = static_cast<T *>(I.v) + W.v_off;
 
   if (it.a0 < 0) {
     // Tip/tilt-only sensor: the sum of its Fried slopes over the valid
     // subapertures is <Gamma^T 1, psi>, which lives on the pupil-edge corners;
-    // one (edge corner, layer) term per thread, one FP64 partial per chunk.
+    // (edge corner, layer) terms, one FP64 partial per chunk of kFwdChunk.
     if (MODE == 2) return;   // data only: the model term is zero
-    const int pair = it.tile * kThreads + tid;
-    const bool on = tid < kThreads && pair < W.n_edge * L;
-    int x0 = 0, y0 = 0, x1 = 0, y1 = 0, N = 1, off = 0;
-    T fx = T(0), fy = T(0), tx = T(0), ty = T(0);
-    if (on) {
+    constexpr int U = kFwdChunk / kFwdThreads;
+    int at[U][4];
+    T fx[U], fy[U], tx[U], ty[U];
+    bool on[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int pair = it.tile * kFwdChunk + u * kFwdThreads + tid;
+      on[u] = tid < kFwdThreads && pair < W.n_edge * L;
+      if (!on[u]) continue;
       const int e = pair / L, l = pair - e * L;
       const int c = I.edge_idx[W.edge_off + e];
       const int a = c % nc, b = c / nc;
       const T *et = static_cast<const T *>(I.edge_t) + 2 * (W.edge_off + e);
-      const T *pf = static_cast<const T *>(I.pos_f);
-      const int po = I.pos_off[it.wfs * L + l];
-      N = I.layers[l].N;
-      off = I.layers[l].off;
-      x0 = I.pos_i0[po + a];
-      y0 = I.pos_i0[po + nc + b];
-      fx = pf[po + a];
-      fy = pf[po + nc + b];
-      x1 = (x0 + 1) & (N - 1);
-      y1 = (y0 + 1) & (N - 1);
-      tx = et[0];
-      ty = et[1];
+      const int po = 2 * l * nc, N = I.layers[l].N, off = I.layers[l].off;
+      const int x0 = pi[po + a], y0 = pi[po + nc + b];
+      const int x1 = (x0 + 1) & (N - 1), y1 = (y0 + 1) & (N - 1);
+      at[u][0] = off + y0 * N + x0;
+      at[u][1] = off + y0 * N + x1;
+      at[u][2] = off + y1 * N + x0;
+      at[u][3] = off + y1 * N + x1;
+      fx[u] = pf[po + a];
+      fy[u] = pf[po + nc + b];
+      tx[u] = et[0];
+      ty[u] = et[1];
     }
     pdl_wait();
     Acc<T> ax, ay;
-    if (on) {
-      const T *p = phi + off;
-      const T v00 = p[y0 * N + x0], v01 = p[y0 * N + x1];
-      const T v10 = p[y1 * N + x0], v11 = p[y1 * N + x1];
-      const T ps = (T(1) - fy) * ((T(1) - fx) * v00 + fx * v01) + fy * ((T(1) - fx) * v10 + fx * v11);
-      ax.add_prod(tx, ps);
-      ay.add_prod(ty, ps);
-    }
-    store_tile_partial(I.part + W.part_off + 2 * it.tile, ax, ay);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (on[u]) {
+        const T v00 = phi[at[u][0]], v01 = phi[at[u][1]];
+        const T v10 = phi[at[u][2]], v11 = phi[at[u][3]];
+        const T ps = lerp(fy[u], lerp(fx[u], v00, v01), lerp(fx[u], v10, v11));
+        ax.add_prod(tx[u], ps);
+        ay.add_prod(ty[u], ps);
+      }
+    store_tile_partial(part + 2 * it.tile, ax, ay);
     return;
   }
 
   // stage this tile's corner->node tables for every layer (constant data)
-  int *s_N = reinterpret_cast<int *>(fsm);
+  FwdRow<T> *s_row = reinterpret_cast<FwdRow<T> *>(fsm);
+  T *s_fx = reinterpret_cast<T *>(s_row + L * kFwdPsi);
+  int *s_x0 = reinterpret_cast<int *>(s_fx + L * kFwdLanes);
+  int *s_N = s_x0 + L * kFwdLanes;
   int *s_off = s_N + L;
-  int *s_x0 = s_off + L;
-  int *s_y0 = s_x0 + L * kHalo;
-  T *s_fx = reinterpret_cast<T *>(fsm + ((sizeof(int) * (2 * L + 2 * L * kHalo) + 15) & ~size_t(15)));
-  T *s_fy = s_fx + L * kHalo;
   const int a0 = it.a0, b0 = it.b0;
-  {
-    const T *pf = static_cast<const T *>(I.pos_f);
-    for (int idx = tid; idx < L * kHalo; idx += blockDim.x) {
-      const int l = idx / kHalo, u = idx - l * kHalo;
-      const int po = I.pos_off[it.wfs * L + l];
-      const int a = min(max(a0 - 1 + u, 0), nc - 1), b = min(max(b0 - 1 + u, 0), nc - 1);
-      s_x0[idx] = I.pos_i0[po + a];
-      s_fx[idx] = pf[po + a];
-      s_y0[idx] = I.pos_i0[po + nc + b];
-      s_fy[idx] = pf[po + nc + b];
+  if (MODE != 2) {
+    for (int idx = tid; idx < L * kFwdLanes; idx += nt) {
+      const int l = idx / kFwdLanes, u = idx - l * kFwdLanes;
+      const int a = 2 * l * nc + min(max(a0 - 1 + u, 0), nc - 1);
+      s_x0[idx] = pi[a];
+      s_fx[idx] = pf[a];
     }
-    for (int l = tid; l < L; l += blockDim.x) {
+    for (int idx = tid; idx < L * kFwdPsi; idx += nt) {
+      const int l = idx / kFwdPsi, w = idx - l * kFwdPsi;
+      const int b = 2 * l * nc + nc + min(max(b0 - 1 + w, 0), nc - 1);
+      s_row[idx].r0 = pi[b] * I.layers[l].N;
+      s_row[idx].f = pf[b];
+    }
+    for (int l = tid; l < L; l += nt) {
       s_N[l] = I.layers[l].N;
       s_off[l] = I.layers[l].off;
     }
   }
-  __syncthreads();
   const unsigned char *act = I.active + W.act_off;
   const int *sidx = I.sub_idx + W.sub_off;
-  pdl_wait();
+  const int lane = tid & 31, warp = tid >> 5;
+  // the slope indices of step 2 (constant: before the dependency wait)
+  constexpr int kSubRounds = (kFwdRows + kFwdThreads / 32) / (kFwdThreads / 32);
+  int sj[kSubRounds];
+#pragma unroll
+  for (int q = 0; q < kSubRounds; ++q) {
+    const int w = warp + q * (kFwdThreads / 32), a = a0 - 1 + lane, b = b0 - 1 + w;
+    sj[q] = tid < kFwdThreads && lane <= kFwdCols && w <= kFwdRows && a >= 0 && b >= 0 && a < n && b < n
+                ? sidx[b * n + a]
+                : -1;
+  }
   // 1. psi on the tile's corners plus a one-corner halo
-  for (int idx = tid; idx < kHalo * kHalo; idx += blockDim.x) {
-    const int u = idx % kHalo, w = idx / kHalo;
-    const int a = a0 - 1 + u, b = b0 - 1 + w;
-    T val = T(0);
-    if (MODE != 2 && a >= 0 && b >= 0 && a < nc && b < nc && act[b * nc + a]) {
-      // four layers' loads in flight at a time; the sum keeps the layer order
-      for (int l0 = 0; l0 < L; l0 += 4) {
-        T v00[4], v01[4], v10[4], v11[4], fx[4], fy[4];
+  {
+    const int a = a0 - 1 + lane, w = warp * RS;
+    bool on[RS];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int l = l0 + j < L ? l0 + j : L - 1;
-          const int N = s_N[l];
-          const int x0 = s_x0[l * kHalo + u], y0 = s_y0[l * kHalo + w];
-          fx[j] = s_fx[l * kHalo + u];
-          fy[j] = s_fy[l * kHalo + w];
-          const int x1 = (x0 + 1) & (N - 1), y1 = (y0 + 1) & (N - 1);
-          const T *p = phi + s_off[l];
-          v00[j] = p[y0 * N + x0];
-          v01[j] = p[y0 * N + x1];
-          v10[j] = p[y1 * N + x0];
-          v11[j] = p[y1 * N + x1];
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (l0 + j < L)
-            val += (T(1) - fy[j]) * ((T(1) - fx[j]) * v00[j] + fx[j] * v01[j]) +
-                   fy[j] * ((T(1) - fx[j]) * v10[j] + fx[j] * v11[j]);
-      }
+    for (int j = 0; j < RS; ++j) {
+      const int b = b0 - 1 + w + j;
+      on[j] = MODE != 2 && a >= 0 && b >= 0 && a < nc && b < nc && act[b * nc + a];
     }
-    s_psi[w][u] = val;
+    __syncthreads();
+    pdl_wait();
+    T val[RS];
+    if (MODE != 2) trace_strip<T, RS>(phi, L, w, s_N, s_off, s_x0, s_fx, s_row, val);
+#pragma unroll
+    for (int j = 0; j < RS; ++j) s_psi[w + j][lane] = on[j] ? val[j] : T(0);
   }
   __syncthreads();
-  // 2. weighted slopes of the subapertures the tile's corners touch
+  // 2. weighted slopes of the subapertures the tile's corners touch: four warps, one lane per column
   Acc<T> sx_acc, sy_acc, qx_acc, qy_acc;
   const T isg = sizeof(T) == 4 ? T(W.inv_sigma2_f) : T(W.inv_sigma2);   // no FP64 conversion in FP32
   // spot elongation: the block sigma^2 (I + tau g g^T) is inverted in closed
@@ -239,12 +331,13 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT == kFwdThreads ? 2 : 
   const T el_cx = EL ? T(0.5 - 0.5 * n) * el_d - T(W.el_lx) : T(0);
   const T el_cy = EL ? T(0.5 - 0.5 * n) * el_d - T(W.el_ly) : T(0);
   const bool four = EL && tile_partials(W) == 4;
-  for (int idx = tid; tid < kThreads && idx < (kFwdTile + 1) * (kFwdTile + 1); idx += kThreads) {
-    const int u = idx % (kFwdTile + 1), w = idx / (kFwdTile + 1);
-    const int a = a0 - 1 + u, b = b0 - 1 + w;
-    T ex = T(0), ey = T(0);
-    if (a >= 0 && b >= 0 && a < n && b < n) {
-      const int j = sidx[b * n + a];
+  if (tid < kFwdThreads && lane <= kFwdCols) {
+    const int u = lane, a = a0 - 1 + u;
+#pragma unroll
+    for (int q = 0; q < kSubRounds; ++q) {
+      const int w = warp + q * (kFwdThreads / 32), b = b0 - 1 + w, j = sj[q];
+      if (w > kFwdRows) break;
+      T ex = T(0), ey = T(0);
       if (j >= 0) {
         const T p00 = s_psi[w][u], p10 = s_psi[w][u + 1];
         const T p01 = s_psi[w + 1][u], p11 = s_psi[w + 1][u + 1];
@@ -276,30 +369,31 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT == kFwdThreads ? 2 : 
           }
         }
       }
+      s_ex[w][u] = ex;
+      s_ey[w][u] = ey;
     }
-    s_ex[w][u] = ex;
-    s_ey[w][u] = ey;
   }
   __syncthreads();
   // 3. Gamma^T: each corner gathers its four neighbouring subapertures
-  T *v = static_cast<T *>(I.v) + W.v_off;
-  if (tid < kFwdTile * kFwdTile) {
-    const int u = tid % kFwdTile, w = tid / kFwdTile;
-    const int a = a0 + u, b = b0 + w;
-    if (a < nc && b < nc) {
-      const T val = T(0.5) * (s_ex[w + 1][u] + s_ex[w][u] - s_ex[w + 1][u + 1] - s_ex[w][u + 1]) +
-                    T(0.5) * (-s_ey[w + 1][u] + s_ey[w][u] - s_ey[w + 1][u + 1] + s_ey[w][u + 1]);
-      v[b * nc + a] = val;
+  if (lane < kFwdCols) {
+    const int u = lane, a = a0 + u;
+    for (int w = warp; w < kFwdRows; w += nt >> 5) {
+      const int b = b0 + w;
+      if (a < nc && b < nc) {
+        const T val = T(0.5) * (s_ex[w + 1][u] + s_ex[w][u] - s_ex[w + 1][u + 1] - s_ex[w][u + 1]) +
+                      T(0.5) * (-s_ey[w + 1][u] + s_ey[w][u] - s_ey[w + 1][u + 1] + s_ey[w][u + 1]);
+        v[b * nc + a] = val;
+      }
     }
   }
   if (W.kind != kRemoveTT) return;
   // 4. tip/tilt removal: this tile's sums of z (the consumer forms the means)
   if (four) {
-    store_tile_partial(I.part + W.part_off + 4 * it.tile, sx_acc, sy_acc);
+    store_tile_partial(part + 4 * it.tile, sx_acc, sy_acc);
     __syncthreads();   // warp 0 has read the reduction scratch before it is reused
-    store_tile_partial(I.part + W.part_off + 4 * it.tile + 2, qx_acc, qy_acc);
+    store_tile_partial(part + 4 * it.tile + 2, qx_acc, qy_acc);
   } else {
-    store_tile_partial(I.part + W.part_off + 2 * it.tile, sx_acc, sy_acc);
+    store_tile_partial(part + 2 * it.tile, sx_acc, sy_acc);
   }
 }
 
@@ -1427,18 +1521,18 @@ cudaError_t allow_type() {
   if (e == cudaSuccess) e = allow_lf<T, 4>();
   if (e == cudaSuccess) e = allow_lf<T, 6>();
   if (e == cudaSuccess) e = allow_lf<T, 8>();
-  const void *fwd[12] = {reinterpret_cast<const void *>(k_forward<T, 0, false, kFwdThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, false, kFwdThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, false, kFwdThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 0, true, kFwdThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, true, kFwdThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, true, kFwdThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 0, false, kThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, false, kThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, false, kThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 0, true, kThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, true, kThreads>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, true, kThreads>)};
+  const void *fwd[12] = {reinterpret_cast<const void *>(k_forward<T, 0, false, 1>),
+                         reinterpret_cast<const void *>(k_forward<T, 1, false, 1>),
+                         reinterpret_cast<const void *>(k_forward<T, 2, false, 1>),
+                         reinterpret_cast<const void *>(k_forward<T, 0, true, 1>),
+                         reinterpret_cast<const void *>(k_forward<T, 1, true, 1>),
+                         reinterpret_cast<const void *>(k_forward<T, 2, true, 1>),
+                         reinterpret_cast<const void *>(k_forward<T, 0, false, 4>),
+                         reinterpret_cast<const void *>(k_forward<T, 1, false, 4>),
+                         reinterpret_cast<const void *>(k_forward<T, 2, false, 4>),
+                         reinterpret_cast<const void *>(k_forward<T, 0, true, 4>),
+                         reinterpret_cast<const void *>(k_forward<T, 1, true, 4>),
+                         reinterpret_cast<const void *>(k_forward<T, 2, true, 4>)};
   for (int i = 0; i < 12 && e == cudaSuccess; ++i)
     e = cudaFuncSetAttribute(fwd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxForwardSmem);
   return e;
@@ -1513,7 +1607,7 @@ cudaError_t configure_kernels() {
 }
 
 size_t forward_smem(int n_layers, int precision) {
-  return fwd_table_bytes(n_layers, precision ? 8 : 4);
+  return precision ? fwd_table_bytes<double>(n_layers) : fwd_table_bytes<float>(n_layers);
 }
 
 cudaError_t launch_synthesis(int precision, int src, int lf, int flags, const InstDev *insts,
@@ -1530,31 +1624,36 @@ cudaError_t launch_analysis(int precision, int src, int epi, int lf, int flags, 
                         : anal_t<double>(src, epi, lf, flags, insts, items, n_clusters, C, smem, io, s);
 }
 
-template <typename T, bool EL, int NT>
-cudaError_t fwd_nt(int mode, dim3 g, size_t sm, cudaStream_t s, const InstDev *insts, const FwdItem *items,
+template <typename T, bool EL, int RS>
+cudaError_t fwd_rs(int mode, dim3 g, size_t sm, cudaStream_t s, const InstDev *insts, const FwdItem *items,
                    const IoArgs &io) {
-  if (mode == 0) return launch_ex(k_forward<T, 0, EL, NT>, g, NT, 0, sm, s, insts, items, io);
-  if (mode == 1) return launch_ex(k_forward<T, 1, EL, NT>, g, NT, 0, sm, s, insts, items, io);
-  return launch_ex(k_forward<T, 2, EL, NT>, g, NT, 0, sm, s, insts, items, io);
+  constexpr int nt = kFwdThreads * 4 / RS;
+  if (mode == 0) return launch_ex(k_forward<T, 0, EL, RS>, g, nt, 0, sm, s, insts, items, io);
+  if (mode == 1) return launch_ex(k_forward<T, 1, EL, RS>, g, nt, 0, sm, s, insts, items, io);
+  return launch_ex(k_forward<T, 2, EL, RS>, g, nt, 0, sm, s, insts, items, io);
 }
 
 template <typename T, bool EL>
-cudaError_t fwd_t(int mode, dim3 g, int nt, size_t sm, cudaStream_t s, const InstDev *insts,
-                  const FwdItem *items, const IoArgs &io) {
-  return nt == kFwdThreads ? fwd_nt<T, EL, kFwdThreads>(mode, g, sm, s, insts, items, io)
-                           : fwd_nt<T, EL, kThreads>(mode, g, sm, s, insts, items, io);
+cudaError_t fwd_t(int mode, dim3 g, size_t sm, cudaStream_t s, const InstDev *insts, const FwdItem *items,
+                  const IoArgs &io) {
+  return g.x <= kFwdSmallLaunch ? fwd_rs<T, EL, 1>(mode, g, sm, s, insts, items, io)
+                                : fwd_rs<T, EL, 4>(mode, g, sm, s, insts, items, io);
 }
 
 cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, const InstDev *insts,
                            const FwdItem *items, int n_items, const IoArgs &io, cudaStream_t s) {
   const dim3 g(n_items);
-  const int nt = n_items <= kFwdSmallLaunch ? kFwdThreads : kThreads;
-  const size_t sm = forward_smem(max_layers, precision);
+  // A small launch asks for more shared memory than its tables need: with 64 KB per CTA no two of
+  // the analysis kernel's CTAs (about 100 KB) start on one SM beside a forward CTA while other SMs
+  // have none (programmatic launch places them early).  E-ELT frame, us by KB per CTA: 420 (none),
+  // 414 (64), 414 (80), 419 (100), 434 (120).
+  const size_t need = forward_smem(max_layers, precision);
+  const size_t sm = n_items <= kFwdSmallLaunch && need < kFwdSmallSmem ? kFwdSmallSmem : need;
   if (precision == 0)
-    return elong ? fwd_t<float, true>(mode, g, nt, sm, s, insts, items, io)
-                 : fwd_t<float, false>(mode, g, nt, sm, s, insts, items, io);
-  return elong ? fwd_t<double, true>(mode, g, nt, sm, s, insts, items, io)
-               : fwd_t<double, false>(mode, g, nt, sm, s, insts, items, io);
+    return elong ? fwd_t<float, true>(mode, g, sm, s, insts, items, io)
+                 : fwd_t<float, false>(mode, g, sm, s, insts, items, io);
+  return elong ? fwd_t<double, true>(mode, g, sm, s, insts, items, io)
+               : fwd_t<double, false>(mode, g, sm, s, insts, items, io);
 }
 
 cudaError_t launch_update(int precision, int flags, const InstDev *insts, const UpdItem *items,

@@ -8,7 +8,9 @@
 namespace tomo {
 
 constexpr int kMaxTransformSmem = 220 * 1024;   // opt-in dynamic shared memory of the transforms
-constexpr int kMaxForwardSmem = 150 * 1024;     // staged corner tables of the forward kernel
+// Layers whose corner tables the forward kernel stages (FP32, FP64 plans).
+constexpr int kMaxForwardLayers[2] = {518, 349};
+constexpr int kMaxForwardSmem = 204 * 1024;     // their tables
 constexpr size_t kTwoPerSmSmem = 108 * 1024;   // dynamic shared memory that lets two CTAs share an SM
 
 // Dynamic shared memory of k_forward for `n_layers` layers.
