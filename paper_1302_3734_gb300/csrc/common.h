@@ -28,6 +28,7 @@ constexpr int kUpdMaxBlocks = 608; // update CTAs per instance at most (four per
 constexpr int kMaxTapsNode = 4;    // corners per axis whose bilinear taps reach one node
 constexpr int kPassRows = 8;       // half-rows of a level one CTA of a streamed transform pass covers
 constexpr int kPassThreads = 512;  // threads per CTA of the streamed transform kernels
+constexpr int kDwtThreads = 128;   // threads per CTA of a streamed analysis pass (kPassRows half-rows)
 constexpr int kCoarseMax = 64;     // block side up to which one CTA finishes a layer's transform
 
 enum WfsKind : int { kFull = 0, kRemoveTT = 1, kTTOnly = 2 };

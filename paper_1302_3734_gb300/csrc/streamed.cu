@@ -77,24 +77,54 @@ constexpr int kEmitU = 4;
 // gathered grid in the plan's phi; levels > 1 read the previous low-low block.
 // The low-low part goes to the scratch (or is emitted at k = J); the details
 // are emitted.  One partial pair per CTA.
+//
+// A warp takes 128 input columns (four per lane: two output columns of each
+// half) and walks down its share of the tile's half-rows: per half-row two new
+// input rows, their row transforms from the lane's window of LF + 2 inputs
+// (16-byte loads; the neighbours' overlap hits the L1), then the column sums
+// over the last LF row transforms, which stay in registers.  No shared memory
+// and no barrier before the partial sums.  (Staging the tile's rows and their
+// row transforms in shared memory for two barrier-separated passes, one output
+// column per thread, took about four times the instructions.)
+template <typename T>
+struct alignas(16) Quad {
+  T v[4];
+};
+
+template <typename T, int LF>
+struct RowWalk {
+  // row transforms of one input row for the lane's four columns: low outputs
+  // 2q, 2q + 1 and high outputs 2q, 2q + 1, each sum over t in order
+  T l0, l1, h0, h1;
+  static constexpr int NV = (LF + 5) / 4;   // vectors of the window of LF + 2 inputs
+  __device__ __forceinline__ void sums(const Filt<T, LF> &f, const Quad<T> (&w)[NV]) {
+    T lo0 = T(0), hi0 = T(0), lo1 = T(0), hi1 = T(0);
+#pragma unroll
+    for (int t = 0; t < LF; ++t) {
+      lo0 += f.h[t] * w[t >> 2].v[t & 3];
+      hi0 += f.g[t] * w[t >> 2].v[t & 3];
+      lo1 += f.h[t] * w[(t + 2) >> 2].v[(t + 2) & 3];
+      hi1 += f.g[t] * w[(t + 2) >> 2].v[(t + 2) & 3];
+    }
+    l0 = lo0;
+    l1 = lo1;
+    h0 = hi0;
+    h1 = hi1;
+  }
+};
+
 template <typename T, int SRC, int EPI, int LF>
-__global__ void __launch_bounds__(kPassThreads) k_dwt_pass(const InstDev *__restrict__ insts,
-                                                           const PassItem *__restrict__ items, IoArgs io,
-                                                           int k, int flags) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ InstDev sI;
+__global__ void __launch_bounds__(kDwtThreads) k_dwt_pass(const InstDev *__restrict__ insts,
+                                                          const PassItem *__restrict__ items, IoArgs io,
+                                                          int k, int flags) {
   __shared__ T s_dal[kMaxLevels + 1];
   pdl_trigger();
   const PassItem it = items[blockIdx.x];
   if (io.active && !io.active[it.inst]) return;
-  load_inst(&sI, insts + it.inst);
-  const InstDev &I = sI;
+  const InstDev &I = insts[it.inst];
   const LayerDev &L = I.layers[it.layer];
-  const int J = I.J, tid = threadIdx.x, nt = blockDim.x;
+  const int J = I.J, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kDwtThreads / 32;
   const int lgM = L.log2N - (k - 1), M = 1 << lgM, H = M >> 1;
-  constexpr int NR = 2 * kPassRows + LF - 2;
-  T *X = reinterpret_cast<T *>(smem_raw);
-  T *B = X + NR * M;
   if (tid <= J) s_dal[tid] = T(L.dalpha[tid]);
   Filt<T, LF> f;
   f.load(I);
@@ -103,53 +133,76 @@ __global__ void __launch_bounds__(kPassThreads) k_dwt_pass(const InstDev *__rest
   const T *src = k > 1 ? static_cast<const T *>(I.lls) + L.ll_off[k - 1]
                        : (SRC == 0 ? static_cast<const T *>(io.in0[it.inst]) : static_cast<const T *>(I.phi)) + L.off;
   T *ll = k < J ? static_cast<T *>(I.lls) + L.ll_off[k] : nullptr;
+  // columns in groups of 128, the tile's half-rows shared by the warps of a group
+  const int groups = M >> 7, per = max(1, nw / groups), rows = kPassRows / per;
   __syncthreads();
   pdl_wait();
-  // input rows 2 row0 .. 2 row0 + NR - 1 (mod M)
-  stage_rows_async<T>(X, src, M, 2 * it.row0, NR, M, M - 1);
-  cp_async_wait_all();
-  __syncthreads();
-  // row pass (x)
-  row_analysis<T, LF>(f, X, B, NR, lgM, tid, nt);
-  __syncthreads();
-  // column pass (y) and the epilogue, kEmitU outputs per thread at once
-  for (int idx0 = tid; idx0 < kPassRows * M; idx0 += kEmitU * nt) {
-    T lo[kEmitU], hi[kEmitU];
-    typename Emit<T, EPI>::Pre fa[kEmitU], fb[kEmitU];
+  const bool vec = emit.aligned(src);
+  constexpr int NV = RowWalk<T, LF>::NV;
+  for (int unit = warp; unit < groups * per; unit += nw) {
+    const int x0 = (unit % groups) * 128 + 4 * lane, i0 = it.row0 + (unit / groups) * rows;
+    RowWalk<T, LF> row[LF];   // the last LF row transforms
+    auto load = [&](int r, Quad<T> (&w)[NV]) {
+      const T *p = src + static_cast<size_t>(r & (M - 1)) * M;
 #pragma unroll
-    for (int u = 0; u < kEmitU; ++u) {
-      const int idx = idx0 + u * nt;
-      if (idx < kPassRows * M) {
-        const int il = idx >> lgM, x = idx & (M - 1);
-        const int i = it.row0 + il;
-        const T *col = B + 2 * il * M + x;
-        T l = T(0), h = T(0);
-#pragma unroll
-        for (int t = 0; t < LF; ++t) {
-          const T val = col[t * M];
-          l += f.h[t] * val;
-          h += f.g[t] * val;
-        }
-        lo[u] = l;
-        hi[u] = h;
-        if (x >= H || k == J) fa[u] = emit.fetch(i, x, -1);
-        fb[u] = emit.fetch(H + i, x, -1);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kEmitU; ++u) {
-      const int idx = idx0 + u * nt;
-      if (idx < kPassRows * M) {
-        const int il = idx >> lgM, x = idx & (M - 1);
-        const int i = it.row0 + il;
-        if (x < H) {
-          if (k == J) emit.put(i, x, J, lo[u], fa[u]);
-          else ll[i * H + x] = lo[u];
+      for (int c = 0; c < NV; ++c) {
+        const T *q = p + ((x0 + 4 * c) & (M - 1));
+        if (vec) {
+          w[c] = *reinterpret_cast<const Quad<T> *>(q);
         } else {
-          emit.put(i, x, k, lo[u], fa[u]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) w[c].v[e] = q[e];
         }
-        emit.put(H + i, x, k, hi[u], fb[u]);
       }
+    };
+    {
+      Quad<T> w[LF - 2 > 0 ? LF - 2 : 1][NV];
+#pragma unroll
+      for (int t = 0; t < LF - 2; ++t) load(2 * i0 + t, w[t]);
+#pragma unroll
+      for (int t = 0; t < LF - 2; ++t) row[t].sums(f, w[t]);
+    }
+#pragma unroll 1
+    for (int i = i0; i < i0 + rows; ++i) {
+      Quad<T> w[2][NV];
+      load(2 * i + LF - 2, w[0]);
+      load(2 * i + LF - 1, w[1]);
+      const int c = x0 >> 1;   // the lane's output columns c, c + 1 of each half
+      const bool top = k == J;
+      typename Emit<T, EPI>::Pre fl[2], fa[2], fb[2], fc[2];   // low-low (k = J), high-x, high-y, high-high
+      if (top) emit.fetch2(i, c, vec, fl);
+      emit.fetch2(i, H + c, vec, fa);
+      emit.fetch2(H + i, c, vec, fb);
+      emit.fetch2(H + i, H + c, vec, fc);
+      row[LF - 2].sums(f, w[0]);
+      row[LF - 1].sums(f, w[1]);
+      T o[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) o[q] = T(0);
+#pragma unroll
+      for (int t = 0; t < LF; ++t) {
+        o[0] += f.h[t] * row[t].l0;
+        o[1] += f.h[t] * row[t].l1;
+        o[2] += f.h[t] * row[t].h0;
+        o[3] += f.h[t] * row[t].h1;
+        o[4] += f.g[t] * row[t].l0;
+        o[5] += f.g[t] * row[t].l1;
+        o[6] += f.g[t] * row[t].h0;
+        o[7] += f.g[t] * row[t].h1;
+      }
+      if (top) {
+        emit.put2(i, c, J, o[0], o[1], fl, vec);
+      } else if (vec) {
+        store_pair(ll + static_cast<size_t>(i) * H + c, o[0], o[1]);
+      } else {
+        ll[static_cast<size_t>(i) * H + c] = o[0];
+        ll[static_cast<size_t>(i) * H + c + 1] = o[1];
+      }
+      emit.put2(i, H + c, k, o[2], o[3], fa, vec);
+      emit.put2(H + i, c, k, o[4], o[5], fb, vec);
+      emit.put2(H + i, H + c, k, o[6], o[7], fc, vec);
+#pragma unroll
+      for (int t = 0; t + 2 < LF; ++t) row[t] = row[t + 2];
     }
   }
   if (EPI == kEpiPlain) return;
@@ -642,7 +695,7 @@ cudaError_t anal_streamed_e(int flags, const InstDev *insts, const StreamSet &S,
   cudaError_t e = cudaSuccess;
   for (int k = 1; k <= S.kmax && e == cudaSuccess; ++k) {
     if (S.cnt[k] == 0) continue;
-    e = launch_ex(k_dwt_pass<T, SRC, EPI, LF>, dim3(S.cnt[k]), kPassThreads, 0, S.smem_pass, s, insts,
+    e = launch_ex(k_dwt_pass<T, SRC, EPI, LF>, dim3(S.cnt[k]), kDwtThreads, 0, 0, s, insts,
                   S.items + S.off[k], io, k, flags);
   }
   if (e == cudaSuccess)
@@ -670,10 +723,6 @@ cudaError_t allow_streamed_t() {
   TOMO_ALLOW((k_idwt_coarse<T, 1, LF>));                      \
   TOMO_ALLOW((k_idwt_pass<T, 0, LF>));                        \
   TOMO_ALLOW((k_idwt_pass<T, 1, LF>));                        \
-  TOMO_ALLOW((k_dwt_pass<T, 0, kEpiPlain, LF>));              \
-  TOMO_ALLOW((k_dwt_pass<T, 2, kEpiPlain, LF>));              \
-  TOMO_ALLOW((k_dwt_pass<T, 2, kEpiOp, LF>));                 \
-  TOMO_ALLOW((k_dwt_pass<T, 2, kEpiResid, LF>));              \
   TOMO_ALLOW((k_dwt_coarse<T, 0, kEpiPlain, LF>));            \
   TOMO_ALLOW((k_dwt_coarse<T, 2, kEpiPlain, LF>));            \
   TOMO_ALLOW((k_dwt_coarse<T, 2, kEpiOp, LF>));               \

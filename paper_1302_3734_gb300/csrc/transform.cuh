@@ -165,6 +165,22 @@ __device__ __forceinline__ void row_analysis(const Filt<T, LF> &f, const T *X, T
   }
 }
 
+// Two neighbouring elements at once (p aligned to both).
+template <typename T>
+struct alignas(2 * sizeof(T)) Pair {
+  T x, y;
+};
+template <typename T>
+__device__ __forceinline__ void load_pair(const T *p, T &a, T &b) {
+  const Pair<T> v = *reinterpret_cast<const Pair<T> *>(p);
+  a = v.x;
+  b = v.y;
+}
+template <typename T>
+__device__ __forceinline__ void store_pair(T *p, T a, T b) {
+  *reinterpret_cast<Pair<T> *>(p) = {a, b};
+}
+
 // Epilogue of the analysis for one output coefficient.
 enum Epi : int { kEpiPlain = 0, kEpiOp = 1, kEpiResid = 2 };
 
@@ -214,6 +230,61 @@ struct Emit {
       acc0.add_prod(r, z);
       acc1.add_prod(r, r);
     }
+  }
+  // The same for the neighbours (row, col), (row, col + 1), col even, without the
+  // cache; vec: the accesses are aligned for both at once.
+  __device__ __forceinline__ void fetch2(int row, int col, bool vec, Pre (&f)[2]) const {
+    if (!vec) {
+      f[0] = fetch(row, col, -1);
+      f[1] = fetch(row, col + 1, -1);
+      return;
+    }
+    const int idx = off + row * N + col;
+    f[0].a = f[1].a = T(0);
+    f[0].j = f[1].j = T(1);
+    const T *a = EPI == kEpiOp ? P : X;
+    if (EPI == kEpiOp || (EPI == kEpiResid && warm)) load_pair(a + idx, f[0].a, f[1].a);
+    if (EPI == kEpiResid && precond) load_pair(jinv + idx, f[0].j, f[1].j);
+  }
+  __device__ __forceinline__ void put2(int row, int col, int level, T w0, T w1, const Pre (&f)[2], bool vec) {
+    if (!vec) {
+      put(row, col, level, w0, f[0]);
+      put(row, col + 1, level, w1, f[1]);
+      return;
+    }
+    const int idx = off + row * N + col;
+    if (EPI == kEpiPlain) {
+      store_pair(out + idx, w0, w1);
+    } else if (EPI == kEpiOp) {
+      const T q0 = w0 + dalpha[level] * f[0].a, q1 = w1 + dalpha[level] * f[1].a;
+      store_pair(Q + idx, q0, q1);
+      acc0.add_prod(f[0].a, q0);
+      acc0.add_prod(f[1].a, q1);
+    } else {
+      T r0 = w0, r1 = w1;
+      if (warm) {
+        r0 -= dalpha[level] * f[0].a;
+        r1 -= dalpha[level] * f[1].a;
+      } else {
+        store_pair(X + idx, T(0), T(0));
+      }
+      const T z0 = precond ? f[0].j * r0 : r0, z1 = precond ? f[1].j * r1 : r1;
+      store_pair(R + idx, r0, r1);
+      store_pair(Pn + idx, z0, z1);
+      acc0.add_prod(r0, z0);
+      acc0.add_prod(r1, z1);
+      acc1.add_prod(r0, r0);
+      acc1.add_prod(r1, r1);
+    }
+  }
+  // every array that fetch2, put2 and the rows at src use starts on 16 bytes
+  // (the plan's do; a caller's may not)
+  __device__ __forceinline__ bool aligned(const T *src) const {
+    uintptr_t a = reinterpret_cast<uintptr_t>(src);
+    if (EPI == kEpiPlain) a |= reinterpret_cast<uintptr_t>(out);
+    if (EPI == kEpiOp) a |= reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(Q);
+    if (EPI == kEpiResid) a |= reinterpret_cast<uintptr_t>(X);
+    return (a & 15) == 0;
   }
   __device__ __forceinline__ void operator()(int row, int col, int level, T w, int slot) {
     put(row, col, level, w, fetch(row, col, slot));
