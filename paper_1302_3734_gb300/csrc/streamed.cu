@@ -653,7 +653,30 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_idwt_pass(const InstDev *__
   T *out = k > 1 ? static_cast<T *>(I.lls) + L.ll_off[k - 1]
                  : (io.out0[it.inst] ? static_cast<T *>(io.out0[it.inst]) : static_cast<T *>(I.phi)) + L.off;
   const int stride = k > 1 ? M : N;
-  // column synthesis (y): output rows 2b and 2b + 1 from the same half-rows
+  // column synthesis (y): output rows 2b and 2b + 1 from the same half-rows; four
+  // neighbouring columns per thread where the output takes 16-byte stores
+  if (sizeof(T) == 4 && lgM >= 2 && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+    const int lgQ = lgM - 2;
+    for (int idx = tid; idx < (kPassRows << lgQ); idx += nt) {
+      const int b = idx >> lgQ, x = (idx & ((1 << lgQ) - 1)) << 2;
+      const int base = b + HL;
+      Quad<T> even{{T(0), T(0), T(0), T(0)}}, odd{{T(0), T(0), T(0), T(0)}};
+#pragma unroll
+      for (int s = 0; s < LF / 2; ++s) {
+        const Quad<T> xl = *reinterpret_cast<const Quad<T> *>(XL + (base - s) * M + x);
+        const Quad<T> xh = *reinterpret_cast<const Quad<T> *>(XH + (base - s) * M + x);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          even.v[e] += f.h[2 * s] * xl.v[e] + f.g[2 * s] * xh.v[e];
+          odd.v[e] += f.h[2 * s + 1] * xl.v[e] + f.g[2 * s + 1] * xh.v[e];
+        }
+      }
+      T *o = out + (2 * it.row0 + 2 * b) * stride + x;
+      *reinterpret_cast<Quad<T> *>(o) = even;
+      *reinterpret_cast<Quad<T> *>(o + stride) = odd;
+    }
+    return;
+  }
   for (int idx = tid; idx < kPassRows * M; idx += nt) {
     const int b = idx >> lgM, x = idx & (M - 1);
     const int base = b + HL;
