@@ -193,9 +193,9 @@ tomo_status enqueue_solve(tomo_plan *tp, const LaunchSet &L, const void *const *
     io.active = active;
     for (int i = 0; i < L.count; ++i) io.out0[i] = x[i];
     TOMO_TRY(timed(tp, kKindUpd, s, [&] {
-      return launch_update(L.precision, it << kIterShift, L.d_inst, L.upd, L.n_upd, io, s);
-    }, "update"));
-    nk += synthesis_launches(L) + 2 + (L.split ? 1 + anal_launches(L) : 1);
+      return launch_update(L.precision, it << kIterShift, L.d_inst, L.count, L.upd, L.n_upd, io, s);
+    }, "update", update_launches(L.n_upd)));
+    nk += synthesis_launches(L) + 1 + update_launches(L.n_upd) + (L.split ? 1 + anal_launches(L) : 1);
   }
   if (n_kernels) *n_kernels = nk;
   return TOMO_OK;
@@ -863,7 +863,7 @@ tomo_status tomo_plan_get_info(const tomo_plan *p, tomo_plan_info *out) {
   out->cluster_size = H.C;
   const LaunchSet &L = p->ls;
   const int adj = L.split ? 1 + anal_launches(L) : 1;
-  out->kernels_per_iteration = synthesis_launches(L) + 2 + adj;
+  out->kernels_per_iteration = synthesis_launches(L) + 1 + update_launches(L.n_upd) + adj;
   out->kernels_per_solve_base = synthesis_launches(L) + 1 + adj;
   out->gather_separate = L.split;
   out->streamed = L.stream;

@@ -25,6 +25,7 @@ constexpr int kGatherThreads = 512;    // threads per CTA of the separate gather
 constexpr int kMaxGatherSensors = 64;  // dense sensors the separate gather kernel lists
 constexpr int kUpdChunk = 1024;    // coefficients per pass of a vector-update CTA
 constexpr int kUpdMaxBlocks = 608; // update CTAs per instance at most (four per SM of 152 SMs)
+constexpr int kUpdAlphaBlocks = kUpdMaxBlocks;   // update CTAs of a launch above which k_alpha forms alpha first
 constexpr int kMaxTapsNode = 4;    // corners per axis whose bilinear taps reach one node
 constexpr int kPassRows = 8;       // half-rows of a level one CTA of a streamed transform pass covers
 constexpr int kPassThreads = 512;  // threads per CTA of the streamed transform kernels
@@ -42,6 +43,7 @@ enum Scalar : int {
   kRz0 = 0,
   kRz1 = 1,
   kBeta = 2,    // beta of the iteration, stored by the streamed coarse synthesis for its passes
+  kAlpha = 3,   // alpha of the iteration (an element of the plan's type), stored by k_alpha
   kFlag = 5,    // 1 after a breakdown (p.Ap <= 0 or not finite)
   kNumScalars = 8
 };

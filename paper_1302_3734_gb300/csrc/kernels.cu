@@ -1176,7 +1176,45 @@ __device__ __forceinline__ void upd_store(T *X, T *R, int n, int i0, bool vec, c
   }
 }
 
+//
+// The step itself: alpha from the sum p.q of the partials (thread 0 of a CTA).
+// A breakdown (p.Ap <= 0 or a value that is not finite) is recorded when `record`.
 template <typename T>
+__device__ __forceinline__ T step_alpha(const InstDev &I, double pq, double rz, double flag, bool record) {
+  // r = 0 (so p = 0 and p.Ap = 0) means the iterate is already exact: step 0
+  const bool exact = (pq == 0.0 && rz == 0.0);
+  const bool bad = !exact && (!(pq > 0.0) || !isfinite(pq) || !isfinite(rz) || flag != 0.0);
+  if (bad && record) {
+    I.scal[kFlag] = 1.0;
+    if (I.bd_word) *reinterpret_cast<volatile int *>(I.bd_word) = 1;
+  }
+  return T((bad || exact) ? 0.0 : rz / pq);
+}
+
+// alpha of every instance of a big launch, one CTA each, before k_update<T, true>.
+// In a launch of many update CTAs the sum and the division, about 60 FP64 warp
+// instructions per CTA at 16 cycles of the SM's FP64 pipe each, otherwise cost
+// more than the vectors: 64 uneven systems (10332 CTAs), GB300, 90 us an update
+// with a sum per CTA, 62 us with this kernel's.  One wave of CTAs (up to
+// kUpdAlphaBlocks: one E-ELT or 100 m system) is faster without the extra launch
+// (100 m frame 2785 against 2823 us).
+template <typename T>
+__global__ void __launch_bounds__(128) k_alpha(const InstDev *__restrict__ insts, IoArgs io, int flags) {
+  pdl_trigger();
+  if (io.active && !io.active[blockIdx.x]) return;
+  const InstDev &I = insts[blockIdx.x];
+  const int iter = flags >> kIterShift;
+  const double *part = I.part + I.cl_part_off;
+  const int count = I.n_cl_part;
+  double *scal = I.scal;
+  pdl_wait();
+  const double rz = scal[kRz0 + (iter & 1)], flag = scal[kFlag];
+  const double pq = sum_partial(part, count, 0);
+  if (threadIdx.x == 0) *reinterpret_cast<T *>(scal + kAlpha) = step_alpha<T>(I, pq, rz, flag, true);
+}
+
+// PRE: k_alpha has stored alpha; otherwise every CTA forms it.
+template <typename T, bool PRE>
 __global__ void __launch_bounds__(kThreads) k_update(const InstDev *__restrict__ insts,
                                                     const UpdItem *__restrict__ items, IoArgs io,
                                                     int flags) {
@@ -1202,23 +1240,17 @@ __global__ void __launch_bounds__(kThreads) k_update(const InstDev *__restrict__
   bool vec = sizeof(T) == 4 && i0 + 3 < n && aligned;
   T xv[4], rv[4], pv[4], qv[4], jv[4];
   upd_load(X, R, P, Q, Jv, precond, n, i0, vec, xv, rv, pv, qv, jv);
-  {
+  T alpha;
+  if (PRE) {
+    alpha = *reinterpret_cast<const T *>(I->scal + kAlpha);
+  } else {
     const double rz = I->scal[kRz0 + (iter & 1)];
     const double flag = I->scal[kFlag];
     const double pq = sum_partial(I->part + I->cl_part_off, I->n_cl_part, 0);
-    if (threadIdx.x == 0) {
-      // r = 0 (so p = 0 and p.Ap = 0) means the iterate is already exact: step 0
-      const bool exact = (pq == 0.0 && rz == 0.0);
-      const bool bad = !exact && (!(pq > 0.0) || !isfinite(pq) || !isfinite(rz) || flag != 0.0);
-      if (bad && it.blk == 0) {
-        I->scal[kFlag] = 1.0;
-        if (I->bd_word) *reinterpret_cast<volatile int *>(I->bd_word) = 1;
-      }
-      s_alpha = T((bad || exact) ? 0.0 : rz / pq);
-    }
+    if (threadIdx.x == 0) s_alpha = step_alpha<T>(*I, pq, rz, flag, it.blk == 0);
     __syncthreads();
+    alpha = s_alpha;
   }
-  const T alpha = s_alpha;
   // a step of zero (breakdown, or an exact iterate) leaves x and r as they are,
   // even where p or q is not finite: the iterate is frozen
   const bool step = alpha != T(0);
@@ -1656,11 +1688,21 @@ cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, c
                : fwd_t<double, false>(mode, g, sm, s, insts, items, io);
 }
 
-cudaError_t launch_update(int precision, int flags, const InstDev *insts, const UpdItem *items,
-                          int n_items, const IoArgs &io, cudaStream_t s) {
+template <typename T>
+cudaError_t update_t(int flags, const InstDev *insts, int count, const UpdItem *items, int n_items, const IoArgs &io,
+                     cudaStream_t s) {
   const dim3 g(n_items);
-  return precision == 0 ? launch_ex(k_update<float>, g, kThreads, 0, 0, s, insts, items, io, flags)
-                        : launch_ex(k_update<double>, g, kThreads, 0, 0, s, insts, items, io, flags);
+  if (n_items <= kUpdAlphaBlocks) return launch_ex(k_update<T, false>, g, kThreads, 0, 0, s, insts, items, io, flags);
+  const cudaError_t e = launch_ex(k_alpha<T>, dim3(count), 128, 0, 0, s, insts, io, flags);
+  return e != cudaSuccess ? e : launch_ex(k_update<T, true>, g, kThreads, 0, 0, s, insts, items, io, flags);
+}
+
+int update_launches(int n_items) { return n_items <= kUpdAlphaBlocks ? 1 : 2; }
+
+cudaError_t launch_update(int precision, int flags, const InstDev *insts, int count, const UpdItem *items,
+                          int n_items, const IoArgs &io, cudaStream_t s) {
+  return precision == 0 ? update_t<float>(flags, insts, count, items, n_items, io, s)
+                        : update_t<double>(flags, insts, count, items, n_items, io, s);
 }
 
 cudaError_t launch_slopes(int precision, const InstDev *insts, int n_wfs, int max_sub2,

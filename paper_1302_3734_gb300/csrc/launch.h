@@ -57,9 +57,11 @@ cudaError_t configure_gather_kernels();
 cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, const InstDev *insts,
                            const FwdItem *items, int n_items, const IoArgs &io, cudaStream_t s);
 
-// x, r update and the FP64 r.z partials; flags carries the iteration index.
-cudaError_t launch_update(int precision, int flags, const InstDev *insts, const UpdItem *items,
+// x, r update of `count` instances and the FP64 r.z partials; flags carries the iteration
+// index.  update_launches: the kernels one call launches.
+cudaError_t launch_update(int precision, int flags, const InstDev *insts, int count, const UpdItem *items,
                           int n_items, const IoArgs &io, cudaStream_t s);
+int update_launches(int n_items);
 
 // Noise-free measurement (single instance).
 cudaError_t launch_slopes(int precision, const InstDev *insts, int n_wfs, int max_sub2,
