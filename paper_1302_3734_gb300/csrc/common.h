@@ -55,6 +55,7 @@ struct LayerDev {
   int N, log2N;
   int off;                      // offset of this layer in the coefficient / grid vectors
   int cache_kc;                 // transforms cache the coefficients of levels >= cache_kc
+  int coarse, pad_coarse;       // side of the low-low block that CTA 0 of a cluster finishes
   double dalpha[kMaxLevels + 1];  // alpha * D at level k (index k = 1..J)
   double dprior[kMaxLevels + 1];  // D at level k, without alpha
   // Streamed transforms: levels 1..ks-1 run as row-tile passes over the whole
@@ -193,18 +194,31 @@ struct IoArgs {
 TOMO_HD inline int tile_partials(const WfsDev &d) { return (d.elong && d.kind == 1) ? 4 : 2; }
 
 
+// Side of the low-low block from which CTA 0 of a cluster finishes a layer's
+// transform alone: a level over the cluster costs two barriers and a round trip
+// to the neighbours (about 2 us), one of a 32 x 32 block in one CTA less than
+// half of that.  Against S = C (GB300, 10 iterations): one E-ELT frame 416 ->
+// 407 us, one 8 m frame 222 -> 209 us.  At most 32 and N / 2, at least C (a row per CTA), and the
+// block and its row transforms fit one of the two row buffers.
+TOMO_HD inline int transform_coarse_side(int N, int C) {
+  int s = C;
+  while (2 * s <= 32 && 2 * s <= N / 2 && 2 * (2 * s) * (2 * s) <= (N / C + kMaxTaps) * N) s *= 2;
+  return s;
+}
+
 // Shared-memory layout of the transform kernels (elements of T): two row
-// buffers of (N/C + kMaxTaps) x N, two coarse buffers of C x C, then the
-// coefficient cache.
-TOMO_HD inline int transform_cache_offset(int N, int C) {
-  return 2 * (N / C + kMaxTaps) * N + 2 * C * C;
+// buffers of (N/C + kMaxTaps) x N, two coarse buffers of S x S (S the coarse
+// side; when S > C the analysis has them in its second row buffer and the
+// synthesis after the cache), then the coefficient cache.
+TOMO_HD inline int transform_cache_offset(int N, int C, int S) {
+  return 2 * (N / C + kMaxTaps) * N + (S > C ? 0 : 2 * C * C);
 }
 
 // Elements of the coefficient cache of one CTA when levels >= kc are cached
 // (the largest over the cluster's ranks: rank 0 also holds the coarse block).
-TOMO_HD inline int transform_cache_size(int N, int C, int J, int kc) {
+TOMO_HD inline int transform_cache_size(int N, int C, int S, int J, int kc) {
   int kd = 0;
-  while (kd < J && (N >> kd) >= 2 * C) ++kd;
+  while (kd < J && (N >> kd) > S) ++kd;
   int total = 0;
   for (int k = kc < 1 ? 1 : kc; k <= kd; ++k) {
     const int M = N >> (k - 1), Rh = (M / C) >> 1;
@@ -214,7 +228,7 @@ TOMO_HD inline int transform_cache_size(int N, int C, int J, int kc) {
     const int M = N >> (J - 1), Rh = (M / C) >> 1;
     total += Rh * (M >> 1);
   } else {
-    total += C * C;
+    total += S * S;
   }
   return total;
 }

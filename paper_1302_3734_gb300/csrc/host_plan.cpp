@@ -197,22 +197,32 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
     }
     P->C = cluster_request;
   }
-  {
-    // shared memory of the transforms: row buffers, coarse buffers and the
-    // coefficient cache of as many (coarse-first) levels as fit
-    const long long esz = P->precision ? 8 : 4;
-    const long long budget = 220LL * 1024 - 4096;   // opt-in limit minus static shared memory
+  // shared memory of the transforms: row buffers, coarse buffers and the
+  // coefficient cache of as many (coarse-first) levels as fit
+  const long long esz = P->precision ? 8 : 4;
+  const long long budget = 220LL * 1024 - 4096;   // opt-in limit minus static shared memory
+  const long long kTwoPerSm = 108 * 1024;         // two CTAs per SM
+  bool cluster_fits = true;
+  // wide: CTA 0 finishes the levels from transform_coarse_side on, else from side C on
+  auto size_transforms = [&](bool wide) {
     long long need = 0;
-    bool cluster_fits = true;
+    cluster_fits = true;
     for (auto &d : P->layers) {
-      const long long base = transform_cache_offset(d.N, P->C);
+      d.coarse = wide ? transform_coarse_side(d.N, P->C) : P->C;
+      const long long base = transform_cache_offset(d.N, P->C, d.coarse);
       int kc = 1;
-      while (kc <= J && (base + transform_cache_size(d.N, P->C, J, kc)) * esz > budget) ++kc;
-      const long long bytes = (base + transform_cache_size(d.N, P->C, J, kc)) * esz;
+      while (kc <= J && (base + transform_cache_size(d.N, P->C, d.coarse, J, kc)) * esz > budget) ++kc;
+      const long long bytes = (base + transform_cache_size(d.N, P->C, d.coarse, J, kc) +
+                               (d.coarse > P->C ? 2LL * d.coarse * d.coarse : 0)) * esz;
       cluster_fits = cluster_fits && bytes <= budget;
       d.cache_kc = kc;
       need = std::max(need, bytes);
     }
+    return need;
+  };
+  {
+    long long need = size_transforms(true);
+    if (need > kTwoPerSm) need = size_transforms(false);   // (what fits, and how often, stays as with side C)
     P->smem_transform = need;
     // streamed transforms when asked, or when the cluster CTAs cannot share an SM
     // (one cluster per GPC at a time) or do not fit at all
@@ -220,7 +230,7 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
       *err = "transforms must be 0 (choose), 1 (clusters) or 2 (streamed)";
       return TOMO_ERR_ARG;
     }
-    P->stream_tf = transforms == 2 || (transforms == 0 && need > static_cast<long long>(108 * 1024));
+    P->stream_tf = transforms == 2 || (transforms == 0 && need > kTwoPerSm);
     if (!P->stream_tf && !cluster_fits) {
       *err = "layer grids too large for the cluster transform kernels at this precision";
       return TOMO_ERR_UNSUPPORTED;
@@ -669,18 +679,25 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
   }
   {
     const int esz = P->precision ? 8 : 4;
-    const long long budget = 220LL * 1024 - 4096;
     bool fits = true;
-    long long need = 0;
-    for (const auto &d : P->layers) {
-      const long long tr = (transform_cache_offset(d.N, P->C) +
-                            transform_cache_size(d.N, P->C, J, d.cache_kc)) * static_cast<long long>(esz);
-      const StageLayout sl = stage_layout(P->n_dense, d.N, d.N / P->C, P->rec_stride, esz, P->max_tt_entries,
-                                          P->vstage);
-      const long long st = (tr + 15) / 16 * 16 + sl.total;
-      fits = fits && st <= budget;
-      need = std::max(need, st);
+    auto size_analysis = [&]() {
+      long long need = 0;
+      for (const auto &d : P->layers) {
+        const long long tr = (transform_cache_offset(d.N, P->C, d.coarse) +
+                              transform_cache_size(d.N, P->C, d.coarse, J, d.cache_kc)) * static_cast<long long>(esz);
+        const StageLayout sl = stage_layout(P->n_dense, d.N, d.N / P->C, P->rec_stride, esz, P->max_tt_entries,
+                                            P->vstage);
+        need = std::max(need, (tr + 15) / 16 * 16 + sl.total);
+      }
+      return need;
+    };
+    long long need = size_analysis();
+    if (need > kTwoPerSm && !P->stream_tf) {
+      // the coarse side C where the wider one would cost the second CTA of an SM, or the staging
+      P->smem_transform = size_transforms(false);
+      need = size_analysis();
     }
+    fits = need <= budget;
     fits = fits && !P->stream_tf;   // streamed transforms take the gather from its own kernel
     fits = fits && P->max_tt_entries <= 65535;   // the image's 16-bit entry indices
     P->gather_staged = fits ? 1 : 0;

@@ -401,22 +401,24 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
 
 // Coefficients owned by cluster rank c of one layer, and their place in the
 // CTA's shared-memory cache.  Distributed levels k = 1..kd (block side
-// M = N/2^(k-1) >= 2C, R = M/C rows per CTA, Rh = R/2, H = M/2): the high-x
+// M = N/2^(k-1) >= 2S, R = M/C rows per CTA, Rh = R/2, H = M/2): the high-x
 // part of the low-y rows c*Rh + jl and the high-y rows H + c*Rh + jl; then the
 // CTA's low-low rows of level J (kd == J) or, on rank 0, the coarse pyramid
-// block of side C (kd < J).  Levels below cache_kc are read from global memory.
+// block of side S >= C (kd < J).  Levels below cache_kc are read from global memory.
 struct CoefMap {
-  int N, C, J, kd, kc, crank, lgN, lgC;
+  int N, C, S, J, kd, kc, crank, lgN, lgC, lgS;
   int base[kMaxLevels + 3];
-  __device__ void init(int N_, int C_, int J_, int kc_, int crank_) {
+  __device__ void init(int N_, int C_, int S_, int J_, int kc_, int crank_) {
     N = N_;
     C = C_;
+    S = S_;
     J = J_;
     crank = crank_;
     lgN = __ffs(N) - 1;
     lgC = __ffs(C) - 1;
+    lgS = __ffs(S) - 1;
     kd = 0;
-    while (kd < J && (N >> kd) >= 2 * C) ++kd;
+    while (kd < J && (N >> kd) > S) ++kd;
     kc = kc_ < 1 ? 1 : kc_;
     int off = 0;
     for (int k = 1; k <= kd; ++k) {
@@ -431,7 +433,7 @@ struct CoefMap {
       const int M = N >> (J - 1), Rh = (M / C) >> 1;
       off += Rh * (M >> 1);
     } else if (crank == 0) {
-      off += C * C;
+      off += S * S;
     }
     base[kd + 2] = off;
   }
@@ -447,7 +449,7 @@ struct CoefMap {
     return base[k] + (1 << (lrh + lm - 1)) + (jl << lm) + x;
   }
   __device__ int ll(int jl, int x) const { return base[kd + 1] + (jl << (lgM(J) - 1)) + x; }
-  __device__ int coarse(int r, int c) const { return base[kd + 1] + (r << lgC) + c; }
+  __device__ int coarse(int r, int c) const { return base[kd + 1] + (r << lgS) + c; }
   // pyramid position of cache slot q
   __device__ void pos(int q, int &row, int &col) const {
     if (q >= base[kd + 1]) {
@@ -457,8 +459,8 @@ struct CoefMap {
         row = (crank << lrh) + (q2 >> lh);
         col = q2 & ((1 << lh) - 1);
       } else {
-        row = q2 >> lgC;
-        col = q2 & (C - 1);
+        row = q2 >> lgS;
+        col = q2 & (S - 1);
       }
       return;
     }
@@ -646,10 +648,11 @@ __global__ void __launch_bounds__(kAnalysisThreadsMax, 1) k_analysis(const InstD
   const int N = L.N, R0 = N / C, J = I.J, tid = threadIdx.x, nt = blockDim.x;
   T *A = reinterpret_cast<T *>(smem_raw);
   T *B = A + (R0 + kMaxTaps) * N;
-  T *cb = B + (R0 + kMaxTaps) * N;
-  T *cb2 = cb + C * C;
-  T *cache = reinterpret_cast<T *>(smem_raw) + transform_cache_offset(N, C);
-  if (tid == 0) cm.init(N, C, J, L.cache_kc, crank);
+  const int S = L.coarse;
+  T *cb = S > C ? B : B + (R0 + kMaxTaps) * N;
+  T *cb2 = cb + S * S;
+  T *cache = reinterpret_cast<T *>(smem_raw) + transform_cache_offset(N, C, S);
+  if (tid == 0) cm.init(N, C, S, J, L.cache_kc, crank);
   if (tid <= J) s_dal[tid] = T(L.dalpha[tid]);
   Filt<T, LF> f;
   f.load(I);
@@ -673,7 +676,7 @@ __global__ void __launch_bounds__(kAnalysisThreadsMax, 1) k_analysis(const InstD
   const bool staged = SRC == 1;
   bool copies_ok = true;
   if (staged) {
-    const int off = transform_cache_offset(N, C) + transform_cache_size(N, C, J, L.cache_kc);
+    const int off = transform_cache_offset(N, C, S) + transform_cache_size(N, C, S, J, L.cache_kc);
     unsigned char *sb = smem_raw + ((static_cast<size_t>(off) * sizeof(T) + 15) & ~size_t(15));
     st.carve(sb, I.n_dense, N, R0, I);
     if (tid == 0) {
@@ -746,7 +749,7 @@ __global__ void __launch_bounds__(kAnalysisThreadsMax, 1) k_analysis(const InstD
   // overwrites B (the next level's row pass, or the end of the kernel).
   const int lgN = L.log2N, lgC = __ffs(C) - 1;
   int M = N, k = 1;
-  for (; k <= J && M >= 2 * C; ++k, M >>= 1) {
+  for (; k <= J && M > S; ++k, M >>= 1) {
     const int lgM = lgN - (k - 1), lgR = lgM - lgC;
     const int R = M >> lgC, H = M >> 1, Rh = R >> 1;
     if (k > 1) cluster_wait();
@@ -808,12 +811,13 @@ __global__ void __launch_bounds__(kAnalysisThreadsMax, 1) k_analysis(const InstD
   }
   if (k > 1) cluster_wait();   // the next CTAs have read this CTA's halo rows
   if (k <= J) {
-    // coarse levels: the remaining low-low block (side M = C) in CTA 0
-    cluster.sync();   // every CTA's low-low row is written
+    // coarse levels: the remaining low-low block (side M = S) in CTA 0
+    cluster.sync();   // every CTA's low-low rows are written
     if (crank == 0) {
+      const int lgS = __ffs(S) - 1, lgRs = lgS - lgC;   // each CTA holds S / C rows of side S
       for (int idx = tid; idx < M * M; idx += nt) {
-        const int r = idx >> lgC, c = idx & (M - 1);   // M == C here
-        cb[idx] = cluster.map_shared_rank(A, r)[c];   // each CTA holds one row of side M
+        const int r = idx >> lgS, c = idx & (M - 1);
+        cb[idx] = cluster.map_shared_rank(A, r >> lgRs)[((r & ((1 << lgRs) - 1)) << lgS) + c];
       }
     }
     cluster.sync();
@@ -877,10 +881,13 @@ __global__ void __launch_bounds__(kSynthThreads, 1) k_synthesis(const InstDev *_
   const int N = L.N, R0 = N / C, J = I.J, tid = threadIdx.x, nt = blockDim.x;
   T *buf0 = reinterpret_cast<T *>(smem_raw);
   T *buf1 = buf0 + (R0 + kMaxTaps) * N;
-  T *cb = buf1 + (R0 + kMaxTaps) * N;   // low-low of the coarse stage
-  T *cb2 = cb + C * C;                  // column-synthesised block
-  T *cache = reinterpret_cast<T *>(smem_raw) + transform_cache_offset(N, C);
-  if (tid == 0) cm.init(N, C, J, L.cache_kc, crank);
+  const int S = L.coarse;
+  T *cache = reinterpret_cast<T *>(smem_raw) + transform_cache_offset(N, C, S);
+  // low-low of the coarse stage, then its row syntheses (read by the other CTAs while the row
+  // buffers are in use: after the cache when the analysis has them in a row buffer)
+  T *cb = S > C ? cache + transform_cache_size(N, C, S, J, L.cache_kc) : buf1 + (R0 + kMaxTaps) * N;
+  T *cb2 = cb + S * S;
+  if (tid == 0) cm.init(N, C, S, J, L.cache_kc, crank);
   Filt<T, LF> f;
   f.load(I);
   T *out = io.out0[it.inst] ? static_cast<T *>(io.out0[it.inst]) : static_cast<T *>(I.phi);
@@ -1001,8 +1008,8 @@ __global__ void __launch_bounds__(kSynthThreads, 1) k_synthesis(const InstDev *_
           for (int s = 0; s < LF / 2; ++s) {
             const int t = q + 2 * s;
             const int jj = ((j - t) & (M - 1)) >> 1;
-            const T lo = r < H ? cb[r * H + jj] : c3[r * C + jj];
-            const T hi = c3[r * C + H + jj];
+            const T lo = r < H ? cb[r * H + jj] : c3[r * S + jj];
+            const T hi = c3[r * S + H + jj];
             acc += f.hs(q, s) * lo + f.gs(q, s) * hi;
           }
           cb2[r * M + j] = acc;
@@ -1024,9 +1031,9 @@ __global__ void __launch_bounds__(kSynthThreads, 1) k_synthesis(const InstDev *_
       }
     }
     cluster.sync();
-    // level kd: M = 2C, one low-low row per CTA
-    const T *c0 = cluster.map_shared_rank(cb, 0);
-    for (int j = tid; j < C; j += nt) A[j] = c0[crank * C + j];
+    // level kd: M = 2S, S / C low-low rows per CTA
+    const T *c0 = cluster.map_shared_rank(cb, 0) + crank * (S / C) * S;
+    for (int j = tid; j < S / C * S; j += nt) A[j] = c0[j];
   } else {
     const int M = N >> (J - 1), H = M >> 1, Rh = (M / C) >> 1, lgH = __ffs(H) - 1;
     for (int idx = tid; idx < Rh * H; idx += nt) A[idx] = cache[cm.ll(idx >> lgH, idx & (H - 1))];
