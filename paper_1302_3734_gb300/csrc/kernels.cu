@@ -316,7 +316,11 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
     __syncthreads();
     pdl_wait();
     T val[RS];
-    if (MODE != 2) trace_strip<T, RS>(phi, L, w, s_N, s_off, s_x0, s_fx, s_row, val);
+    // (a warp without a corner of the pupil traces none)
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < RS; ++j) any = any || on[j];
+    if (MODE != 2 && __any_sync(0xffffffffu, any)) trace_strip<T, RS>(phi, L, w, s_N, s_off, s_x0, s_fx, s_row, val);
 #pragma unroll
     for (int j = 0; j < RS; ++j) s_psi[w + j][lane] = on[j] ? val[j] : T(0);
   }
