@@ -118,10 +118,11 @@ constexpr int kFwdLanes = kFwdCols + 2, kFwdPsi = kFwdRows + 2;
 
 // Shared memory of the staged corner tables of L layers: per layer the grid
 // side and offset, the columns' node index and fraction, and per corner row
-// (first node row * N, fraction).
+// (first node row, fraction).  Copied asynchronously: one memory latency for
+// all of them, however many layers there are.
 template <typename T>
 struct FwdRow {
-  int r0;
+  int y0;
   T f;
 };
 template <typename T>
@@ -149,27 +150,28 @@ __device__ __forceinline__ void trace_strip(const T *__restrict__ phi, int L, in
   constexpr int kBatch = RS == 1 ? 4 : 2;
   for (int l0 = 0; l0 < L; l0 += kBatch) {
     T v0[kBatch][RS + 1], v1[kBatch][RS + 1], fx[kBatch], fy[kBatch][RS];
-    int r0[kBatch][RS], mask[kBatch];
+    int r0[kBatch][RS];
     bool odd = false;
 #pragma unroll
     for (int q = 0; q < kBatch; ++q) {
       const int l = l0 + q < L ? l0 + q : L - 1;
       const int N = s_N[l], x0 = s_x0[l * kFwdLanes + lane];
       fx[q] = s_fx[l * kFwdLanes + lane];
-      mask[q] = N * N - 1;
+      const int mask = N * N - 1;
+      const int lgN = 31 - __clz(N);
       const T *p0 = phi + s_off[l] + x0, *p1 = phi + s_off[l] + ((x0 + 1) & (N - 1));
       int last = 0;
 #pragma unroll
       for (int j = 0; j < RS; ++j) {
         const FwdRow<T> row = s_row[l * kFwdPsi + w + j];
-        const int r1 = (row.r0 + N) & mask[q];
-        r0[q][j] = row.r0;
+        const int rj = row.y0 << lgN, r1 = (rj + N) & mask;
+        r0[q][j] = rj;
         fy[q][j] = row.f;
         if (j == 0) {
-          v0[q][0] = p0[row.r0];
-          v1[q][0] = p1[row.r0];
+          v0[q][0] = p0[rj];
+          v1[q][0] = p1[rj];
         } else {
-          odd = odd || (row.r0 != last && row.r0 != r0[q][j - 1]);
+          odd = odd || (rj != last && rj != r0[q][j - 1]);
         }
         v0[q][j + 1] = p0[r1];
         v1[q][j + 1] = p1[r1];
@@ -277,15 +279,16 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
     for (int idx = tid; idx < L * kFwdLanes; idx += nt) {
       const int l = idx / kFwdLanes, u = idx - l * kFwdLanes;
       const int a = 2 * l * nc + min(max(a0 - 1 + u, 0), nc - 1);
-      s_x0[idx] = pi[a];
-      s_fx[idx] = pf[a];
+      cp_async_elem(s_x0 + idx, pi + a);
+      cp_async_elem(s_fx + idx, pf + a);
     }
     for (int idx = tid; idx < L * kFwdPsi; idx += nt) {
       const int l = idx / kFwdPsi, w = idx - l * kFwdPsi;
       const int b = 2 * l * nc + nc + min(max(b0 - 1 + w, 0), nc - 1);
-      s_row[idx].r0 = pi[b] * I.layers[l].N;
-      s_row[idx].f = pf[b];
+      cp_async_elem(&s_row[idx].y0, pi + b);
+      cp_async_elem(&s_row[idx].f, pf + b);
     }
+    cp_async_commit();
     for (int l = tid; l < L; l += nt) {
       s_N[l] = I.layers[l].N;
       s_off[l] = I.layers[l].off;
@@ -313,6 +316,7 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
       const int b = b0 - 1 + w + j;
       on[j] = MODE != 2 && a >= 0 && b >= 0 && a < nc && b < nc && act[b * nc + a];
     }
+    cp_async_wait_all();
     __syncthreads();
     pdl_wait();
     T val[RS];
@@ -1220,7 +1224,22 @@ __global__ void __launch_bounds__(128) k_alpha(const InstDev *__restrict__ insts
   double *scal = I.scal;
   pdl_wait();
   const double rz = scal[kRz0 + (iter & 1)], flag = scal[kFlag];
-  const double pq = sum_partial(part, count, 0);
+  // the sum of sum_partial, in its order, with eight loads in flight per lane
+  __shared__ double s_sp[4];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double a = 0.0;
+  for (int q0 = threadIdx.x; q0 < count; q0 += 8 * 128) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = q0 + u * 128 < count ? part[2 * (q0 + u * 128)] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (q0 + u * 128 < count) a += v[u];
+  }
+  a = warp_sum(a);
+  if (lane == 0) s_sp[w] = a;
+  __syncthreads();
+  const double pq = ((s_sp[0] + s_sp[1]) + s_sp[2]) + s_sp[3];
   if (threadIdx.x == 0) *reinterpret_cast<T *>(scal + kAlpha) = step_alpha<T>(I, pq, rz, flag, true);
 }
 
