@@ -30,6 +30,7 @@ constexpr int kMaxTapsNode = 4;    // corners per axis whose bilinear taps reach
 constexpr int kPassRows = 8;       // half-rows of a level one CTA of a streamed transform pass covers
 constexpr int kPassThreads = 512;  // threads per CTA of the streamed transform kernels
 constexpr int kDwtThreads = 128;   // threads per CTA of a streamed analysis pass (kPassRows half-rows)
+constexpr int kIdwtThreads = 128;  // ... and of a streamed synthesis pass
 constexpr int kCoarseMax = 64;     // block side up to which one CTA finishes a layer's transform
 
 enum WfsKind : int { kFull = 0, kRemoveTT = 1, kTTOnly = 2 };
@@ -42,7 +43,8 @@ constexpr int kMaxEdgeSlots = 64;   // sensors with a pupil-edge term
 enum Scalar : int {
   kRz0 = 0,
   kRz1 = 1,
-  kBeta = 2,    // beta of the iteration, stored by the streamed coarse synthesis for its passes
+  kBeta = 2,    // beta of the iteration (an element of the plan's type), stored by the streamed
+                // coarse synthesis for its passes
   kAlpha = 3,   // alpha of the iteration (an element of the plan's type), stored by k_alpha
   kFlag = 5,    // 1 after a breakdown (p.Ap <= 0 or not finite)
   kNumScalars = 8

@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kPassThreads) k_dwt_coarse(const InstDev *__re
 
 // beta = (r.z)_iter / (r.z)_(iter-1) from the update's partials, as k_synthesis
 // forms it (0 at iteration 0 and after a breakdown); record: store (r.z)_iter
-// and beta itself, which the level passes that follow read (stored_beta).
+// and beta itself (in the plan's type), which the level passes that follow read.
 template <typename T>
 __device__ __forceinline__ T streamed_beta(const InstDev &I, int iter, bool record) {
   __shared__ T s_b;
@@ -309,20 +309,9 @@ __device__ __forceinline__ T streamed_beta(const InstDev &I, int iter, bool reco
     s_b = T(beta);
     if (record) {
       I.scal[kRz0 + (iter & 1)] = rz;
-      I.scal[kBeta] = beta;
+      *reinterpret_cast<T *>(I.scal + kBeta) = T(beta);
     }
   }
-  __syncthreads();
-  return s_b;
-}
-
-// beta of the iteration in a level pass: the coarse synthesis kernel, launched
-// before the passes of every streamed synthesis, formed and stored it, so the
-// passes' many CTAs do not each sum the update's partials on the FP64 pipe.
-template <typename T>
-__device__ __forceinline__ T stored_beta(const InstDev &I) {
-  __shared__ T s_b;
-  if (threadIdx.x == 0) s_b = T(I.scal[kBeta]);
   __syncthreads();
   return s_b;
 }
@@ -491,8 +480,16 @@ __global__ void __launch_bounds__(kPassThreads) k_idwt_coarse(const InstDev *__r
 // half-rows [row0, row0 + kPassRows) and writes their updated directions).  The
 // HL = LF/2 - 1 half-rows before the tile are read too.  Output to the scratch
 // (the low-low block of level k - 1) or, k = 1, the output grid.
+//
+// The CTA stages the tile's coefficients in shared memory, each updated once.
+// Then a thread takes four columns of each half of the block (eight output
+// columns) and a strip of the half-rows, walked downwards: per half-row the row
+// syntheses of the low-y and the high-y row from 16-byte windows, and the column
+// synthesis over the last LF/2 half-rows, whose row syntheses stay in registers.
+// One barrier; a strip repeats the row syntheses of HL half-rows, so a tile has
+// at most four strips.
 template <typename T, int SRC, int LF>
-__global__ void __launch_bounds__(kPassThreads, 2) k_idwt_pass(const InstDev *__restrict__ insts,
+__global__ void __launch_bounds__(kIdwtThreads) k_idwt_pass(const InstDev *__restrict__ insts,
                                                             const PassItem *__restrict__ items, IoArgs io,
                                                             int k, int flags) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -508,13 +505,11 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_idwt_pass(const InstDev *__
   const int lgM = L.log2N - (k - 1), M = 1 << lgM, H = M >> 1;
   T *VL = reinterpret_cast<T *>(smem_raw);   // NI low-y rows [LL | HL], then NI high-y rows [LH | HH]
   T *VH = VL + NI * M;
-  T *XL = VH + NI * M;
-  T *XH = XL + NI * M;
   Filt<T, LF> f;
   f.load(I);
   const T *ll = static_cast<const T *>(I.lls) + L.ll_off[k];
   pdl_wait();
-  const T beta = SRC == 1 ? stored_beta<T>(I) : T(0);
+  const T beta = SRC == 1 ? *reinterpret_cast<const T *>(I.scal + kBeta) : T(0);
   const SynthCoef<T, SRC> coef = synth_coef<T, SRC>(I, io, it.inst, flags, beta);
   // the tile's coefficient rows: 16-byte vectors when every source is aligned (the plan's
   // buffers are; a caller's coefficient vector may not be), else kCoefU positions per
@@ -526,6 +521,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_idwt_pass(const InstDev *__
                    ((L.off & (VN - 1)) == 0) && H >= VN;
   if (vec) {
     const int lgMv = lgM - (__ffs(VN) - 1), mv = M / VN;
+#pragma unroll 4
     for (int q = tid; q < NI * mv; q += nt) {
       const int j = q >> lgMv, x = (q & (mv - 1)) * VN;
       const int ii = (it.row0 - HL + j) & (H - 1);
@@ -595,101 +591,80 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_idwt_pass(const InstDev *__
     }
   }
   __syncthreads();
-  // row synthesis (x): outputs 2m and 2m + 1 of a row from the same taps.  VH
-  // follows VL (rows NI.. are the high-y rows) and XH follows XL.
-  const int lgH = lgM - 1;
-  bool rows_done = false;
-  if constexpr (sizeof(T) == 4 && LF <= 10) {
-    if (lgH >= 2) {
-      // FP32: four neighbouring m per thread from the low and high halves'
-      // inputs m - 4 .. m + 3, two 16-byte vectors each (a multiple of four,
-      // so a vector never straddles the periodic wrap), every output's sum in
-      // the order of the scalar form below
-      const int lgQ = lgH - 2;
-      for (int idx = tid; idx < ((2 * NI) << lgQ); idx += nt) {
-        const int r = idx >> lgQ, m0 = (idx & ((1 << lgQ) - 1)) << 2;
-        const T *row = VL + r * M;
-        T lo[8], hi[8];
-        *reinterpret_cast<float4 *>(lo) = *reinterpret_cast<const float4 *>(row + ((m0 - 4) & (H - 1)));
-        *reinterpret_cast<float4 *>(lo + 4) = *reinterpret_cast<const float4 *>(row + m0);
-        *reinterpret_cast<float4 *>(hi) = *reinterpret_cast<const float4 *>(row + H + ((m0 - 4) & (H - 1)));
-        *reinterpret_cast<float4 *>(hi + 4) = *reinterpret_cast<const float4 *>(row + H + m0);
-        T o[8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          T even = T(0), odd = T(0);
-#pragma unroll
-          for (int s = 0; s < LF / 2; ++s) {
-            const T l = lo[4 + u - s], h = hi[4 + u - s];
-            even += f.h[2 * s] * l + f.g[2 * s] * h;
-            odd += f.h[2 * s + 1] * l + f.g[2 * s + 1] * h;
-          }
-          o[2 * u] = even;
-          o[2 * u + 1] = odd;
-        }
-        T *x = XL + r * M + 2 * m0;
-        *reinterpret_cast<float4 *>(x) = *reinterpret_cast<const float4 *>(o);
-        *reinterpret_cast<float4 *>(x + 4) = *reinterpret_cast<const float4 *>(o + 4);
-      }
-      rows_done = true;
-    }
-  }
-  if (!rows_done)
-  for (int idx = tid; idx < 2 * NI * H; idx += nt) {
-    const int r = idx >> lgH, m = idx & (H - 1);
-    const T *row = VL + r * M;
-    T even = T(0), odd = T(0);
-#pragma unroll
-    for (int s = 0; s < LF / 2; ++s) {
-      const int jj = (m - s) & (H - 1);
-      const T lo = row[jj], hi = row[H + jj];
-      even += f.h[2 * s] * lo + f.g[2 * s] * hi;
-      odd += f.h[2 * s + 1] * lo + f.g[2 * s + 1] * hi;
-    }
-    XL[r * M + 2 * m] = even;
-    XL[r * M + 2 * m + 1] = odd;
-  }
-  __syncthreads();
   T *out = k > 1 ? static_cast<T *>(I.lls) + L.ll_off[k - 1]
                  : (io.out0[it.inst] ? static_cast<T *>(io.out0[it.inst]) : static_cast<T *>(I.phi)) + L.off;
   const int stride = k > 1 ? M : N;
-  // column synthesis (y): output rows 2b and 2b + 1 from the same half-rows; four
-  // neighbouring columns per thread where the output takes 16-byte stores
-  if (sizeof(T) == 4 && lgM >= 2 && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
-    const int lgQ = lgM - 2;
-    for (int idx = tid; idx < (kPassRows << lgQ); idx += nt) {
-      const int b = idx >> lgQ, x = (idx & ((1 << lgQ) - 1)) << 2;
-      const int base = b + HL;
-      Quad<T> even{{T(0), T(0), T(0), T(0)}}, odd{{T(0), T(0), T(0), T(0)}};
+  const bool vout = (reinterpret_cast<uintptr_t>(out) & 15) == 0;   // (a caller's grid may not be aligned)
+  // threads of a strip (a power of two), strips of the tile, half-rows of a strip
+  const int lgLanes = lgM - 3, strips = min(4, max(1, kIdwtThreads >> lgLanes)), rows = kPassRows / strips;
+  if ((tid >> lgLanes) >= strips) return;
+  constexpr int NS = LF / 2;
+  auto load4 = [](const T *p, T *v) {
+    const Quad<T> q = *reinterpret_cast<const Quad<T> *>(p);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = q.v[e];
+  };
+  // the eight row syntheses of a staged row from its inputs m0 - 4 .. m0 + 3 of both halves (a
+  // multiple of four, so a window never straddles the periodic wrap)
+  auto row_synth = [&](const T *row, int m0, T *o) {
+    T lo[8], hi[8];
+    const int mp = (m0 - 4) & (H - 1);
+    if (LF > 2) load4(row + mp, lo);
+    load4(row + m0, lo + 4);
+    if (LF > 2) load4(row + H + mp, hi);
+    load4(row + H + m0, hi + 4);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      T even = T(0), odd = T(0);
 #pragma unroll
       for (int s = 0; s < LF / 2; ++s) {
-        const Quad<T> xl = *reinterpret_cast<const Quad<T> *>(XL + (base - s) * M + x);
-        const Quad<T> xh = *reinterpret_cast<const Quad<T> *>(XH + (base - s) * M + x);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          even.v[e] += f.h[2 * s] * xl.v[e] + f.g[2 * s] * xh.v[e];
-          odd.v[e] += f.h[2 * s + 1] * xl.v[e] + f.g[2 * s + 1] * xh.v[e];
-        }
+        const T l = lo[4 + u - s], h = hi[4 + u - s];
+        even += f.h[2 * s] * l + f.g[2 * s] * h;
+        odd += f.h[2 * s + 1] * l + f.g[2 * s + 1] * h;
       }
-      T *o = out + (2 * it.row0 + 2 * b) * stride + x;
-      *reinterpret_cast<Quad<T> *>(o) = even;
-      *reinterpret_cast<Quad<T> *>(o + stride) = odd;
+      o[2 * u] = even;
+      o[2 * u + 1] = odd;
     }
-    return;
-  }
-  for (int idx = tid; idx < kPassRows * M; idx += nt) {
-    const int b = idx >> lgM, x = idx & (M - 1);
-    const int base = b + HL;
-    T even = T(0), odd = T(0);
+  };
+  auto store8 = [&](T *p, const T *v) {
+    if (vout) {
+      *reinterpret_cast<Quad<T> *>(p) = {{v[0], v[1], v[2], v[3]}};
+      *reinterpret_cast<Quad<T> *>(p + 4) = {{v[4], v[5], v[6], v[7]}};
+    } else {
 #pragma unroll
-    for (int s = 0; s < LF / 2; ++s) {
-      const T xl = XL[(base - s) * M + x], xh = XH[(base - s) * M + x];
-      even += f.h[2 * s] * xl + f.g[2 * s] * xh;
-      odd += f.h[2 * s + 1] * xl + f.g[2 * s + 1] * xh;
+      for (int e = 0; e < 8; ++e) p[e] = v[e];
     }
-    T *o = out + (2 * it.row0 + 2 * b) * stride + x;
-    o[0] = even;
-    o[stride] = odd;
+  };
+  for (int m0 = (tid & ((1 << lgLanes) - 1)) << 2; m0 < H; m0 += 4 * kIdwtThreads) {
+    const int j0 = (tid >> lgLanes) * rows;   // the strip's first staged half-row (HL before its own)
+    T xl[NS][8], xh[NS][8];   // the last NS half-rows' row syntheses, half-row j in slot j mod NS
+#pragma unroll 1
+    for (int js = 0; js < rows + HL; js += NS) {
+#pragma unroll
+      for (int u = 0; u < NS; ++u) {
+        const int j = js + u;
+        if (j >= rows + HL) break;
+        row_synth(VL + (j0 + j) * M, m0, xl[u]);
+        row_synth(VH + (j0 + j) * M, m0, xh[u]);
+        if (j < HL) continue;
+        // column synthesis (y): output rows 2b and 2b + 1
+        T even[8], odd[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) even[e] = odd[e] = T(0);
+#pragma unroll
+        for (int s = 0; s < LF / 2; ++s) {
+          const int q = (u - s + NS) % NS;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            even[e] += f.h[2 * s] * xl[q][e] + f.g[2 * s] * xh[q][e];
+            odd[e] += f.h[2 * s + 1] * xl[q][e] + f.g[2 * s + 1] * xh[q][e];
+          }
+        }
+        T *o = out + static_cast<size_t>(2 * (it.row0 + j0 + j - HL)) * stride + 2 * m0;
+        store8(o, even);
+        store8(o + stride, odd);
+      }
+    }
   }
 }
 
@@ -707,8 +682,9 @@ cudaError_t synth_streamed(int src, int flags, const InstDev *insts, const Strea
     if (S.cnt[k] == 0) continue;
     const dim3 g(S.cnt[k]);
     const PassItem *it = S.items + S.off[k];
-    e = src == 0 ? launch_ex(k_idwt_pass<T, 0, LF>, g, kPassThreads, 0, S.smem_pass, s, insts, it, io, k, flags)
-                 : launch_ex(k_idwt_pass<T, 1, LF>, g, kPassThreads, 0, S.smem_pass, s, insts, it, io, k, flags);
+    const size_t smem = S.smem_pass >> k;   // the staged rows: half of pass_smem_elems at the level's block side
+    e = src == 0 ? launch_ex(k_idwt_pass<T, 0, LF>, g, kIdwtThreads, 0, smem, s, insts, it, io, k, flags)
+                 : launch_ex(k_idwt_pass<T, 1, LF>, g, kIdwtThreads, 0, smem, s, insts, it, io, k, flags);
   }
   return e;
 }
