@@ -546,7 +546,6 @@ tomo_status tomo_plan_create_ex(const tomo_geometry *g, const tomo_plan_options 
   }
   for (const auto &w : H.wfs) {
     p->nc_max = std::max(p->nc_max, w.nc);
-    p->max_sub2 = std::max(p->max_sub2, w.n * w.n);
   }
 
   // ---- arena layout: tables (uploaded) then workspace (zeroed)
@@ -1005,7 +1004,8 @@ tomo_status tomo_layers_to_slopes(tomo_plan *p, const void *d_layers, void *d_sl
   io.in0[0] = d_layers;
   io.out0[0] = d_slopes;
   return timed(p, kKindOther, s, [&] {
-    return launch_slopes(p->ls.precision, p->d_inst, p->hp.n_wfs, p->max_sub2, io, s);
+    const LaunchSet &L = p->ls;
+    return launch_forward(L.precision, 3, L.max_layers, 0, L.d_inst, L.fwd, L.n_fwd, io, s);
   }, "slopes");
 }
 

@@ -459,11 +459,23 @@ __global__ void __launch_bounds__(kFitRmsThreads) k_fit_rms(FitDev F, double *__
   const T *u = static_cast<const T *>(F.u) + static_cast<size_t>(j) * nn;
   pdl_wait();
   Acc<T> s1, s2;
-  for (int c = threadIdx.x; c < nn; c += blockDim.x)
-    if (F.act[c]) {
-      s1.add(u[c]);
-      s2.add_prod(u[c], u[c]);
+  // eight corners' loads at a time (the field is read whether the corner counts or not)
+  for (int c0 = threadIdx.x; c0 < nn; c0 += 8 * blockDim.x) {
+    T v[8];
+    bool on[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int c = min(c0 + q * static_cast<int>(blockDim.x), nn - 1);
+      on[q] = c0 + q * static_cast<int>(blockDim.x) < nn && F.act[c];
+      v[q] = u[c];
     }
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (on[q]) {
+        s1.add(v[q]);
+        s2.add_prod(v[q], v[q]);
+      }
+  }
   const double2 v = block_sum2(s1, s2);
   if (threadIdx.x == 0) {
     const double m = v.x / F.n_points, q = v.y / F.n_points;
@@ -478,23 +490,43 @@ template <typename T>
 __device__ __forceinline__ T sensor_mirror(const FitDev &F, const T *__restrict__ cmd, int tab, int nc, int a,
                                            int b) {
   const T *fx = static_cast<const T *>(F.sfx), *fy = static_cast<const T *>(F.sfy);
+  // every mirror's taps, then every mirror's commands, are requested before any is used (the
+  // indices are clamped; a tap beyond the mirror is not added)
+  int x0[kMaxDm], y0[kMaxDm];
+  T wx1[kMaxDm], wy1[kMaxDm], v[kMaxDm][2][2];
+#pragma unroll
+  for (int k = 0; k < kMaxDm; ++k) {
+    const int o = tab + min(k, F.n_dm - 1) * nc;
+    x0[k] = F.sx0[o + a];
+    y0[k] = F.sy0[o + b];
+    wx1[k] = fx[o + a];
+    wy1[k] = fy[o + b];
+  }
+#pragma unroll
+  for (int k = 0; k < kMaxDm; ++k) {
+    if (k >= F.n_dm) break;
+    const int n = F.dm_n[k];
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+      for (int dx = 0; dx < 2; ++dx)
+        v[k][dy][dx] = cmd[F.dm_off[k] + min(max(y0[k] + dy, 0), n - 1) * n + min(max(x0[k] + dx, 0), n - 1)];
+  }
   T psi = T(0);
 #pragma unroll
   for (int k = 0; k < kMaxDm; ++k) {
     if (k >= F.n_dm) break;
-    const int n = F.dm_n[k], o = tab + k * nc;
-    const int x0 = F.sx0[o + a], y0 = F.sy0[o + b];
-    const T wx1 = fx[o + a], wy1 = fy[o + b];
-    const T wx[2] = {T(1) - wx1, wx1}, wy[2] = {T(1) - wy1, wy1};
+    const int n = F.dm_n[k];
+    const T wx[2] = {T(1) - wx1[k], wx1[k]}, wy[2] = {T(1) - wy1[k], wy1[k]};
 #pragma unroll
     for (int dy = 0; dy < 2; ++dy) {
-      const int iy = y0 + dy;
+      const int iy = y0[k] + dy;
       if (iy < 0 || iy >= n) continue;
       T row = T(0);
 #pragma unroll
       for (int dx = 0; dx < 2; ++dx) {
-        const int ix = x0 + dx;
-        if (ix >= 0 && ix < n) row += wx[dx] * cmd[F.dm_off[k] + iy * n + ix];
+        const int ix = x0[k] + dx;
+        if (ix >= 0 && ix < n) row += wx[dx] * v[k][dy][dx];
       }
       psi += wy[dy] * row;
     }

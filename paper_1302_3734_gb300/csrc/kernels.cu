@@ -64,30 +64,14 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 }
 
 
-// psi at corner (a, b) of sensor m: sum over layers of the bilinear
-// interpolation of phi_l at the corner's traced position (Sec. 2.1, P_m).
-template <typename T>
-__device__ __forceinline__ T trace_corner(const InstDev &I, int m, int nc, const T *phi, int a,
-                                          int b) {
-  const T *pf = static_cast<const T *>(I.pos_f);
-  T acc = T(0);
-  for (int l = 0; l < I.n_layers; ++l) {
-    const int N = I.layers[l].N, off = I.layers[l].off;
-    const int po = I.pos_off[m * I.n_layers + l];
-    const int x0 = I.pos_i0[po + a], y0 = I.pos_i0[po + nc + b];
-    const T fx = pf[po + a], fy = pf[po + nc + b];
-    const int x1 = (x0 + 1) & (N - 1), y1 = (y0 + 1) & (N - 1);
-    const T *p = phi + off;
-    const T v00 = p[y0 * N + x0], v01 = p[y0 * N + x1];
-    const T v10 = p[y1 * N + x0], v11 = p[y1 * N + x1];
-    acc += (T(1) - fy) * ((T(1) - fx) * v00 + fx * v01) + fy * ((T(1) - fx) * v10 + fx * v11);
-  }
-  return acc;
-}
-
 // ------------------------------------------------------------ k_forward
 // MODE 0: operator, z = Gamma P phi.  MODE 1: residual, z = s - Gamma P phi.
-// MODE 2: data only, z = s (phi = 0).  Writes the corner field
+// MODE 2: data only, z = s (phi = 0).  MODE 3: the noise-free measurement A phi
+// itself (eq. atm_tomo) into io.out0: the slopes, and a tip/tilt-only sensor's
+// two means (by its first chunk's CTA alone); nothing of the plan is written.
+// (Four corners traced per subaperture, layer after layer, took 19 us on the
+// E-ELT system, cold on GB300; these tiles 12.)
+// Otherwise writes the corner field
 // v_m = Gamma_m^T sigma^-2 z_m and, with tip/tilt removal, each tile's sums of z
 // (the analysis subtracts the means on the pupil edge, Sec. 4.3 eq. widehatc).
 // A tip/tilt-only sensor writes its weighted mean slopes (e_x, e_y).
@@ -228,6 +212,52 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
     // subapertures is <Gamma^T 1, psi>, which lives on the pupil-edge corners;
     // (edge corner, layer) terms, one FP64 partial per chunk of kFwdChunk.
     if (MODE == 2) return;   // data only: the model term is zero
+    if constexpr (MODE == 3) {
+      if (it.tile != 0) return;
+      pdl_wait();
+      Acc<T> ax, ay;
+      constexpr int kBatch = 5;   // layers whose loads a thread issues together
+      for (int e = tid; e < W.n_edge; e += nt) {
+        const int c = I.edge_idx[W.edge_off + e], a = c % nc, b = c / nc;
+        const T *et = static_cast<const T *>(I.edge_t) + 2 * (W.edge_off + e);
+        const T tx = et[0], ty = et[1];
+        T ps = T(0);
+        for (int l0 = 0; l0 < L; l0 += kBatch) {
+          T v00[kBatch], v01[kBatch], v10[kBatch], v11[kBatch], fx[kBatch], fy[kBatch];
+          int x0[kBatch], y0[kBatch];
+#pragma unroll
+          for (int q = 0; q < kBatch; ++q) {
+            const int po = 2 * min(l0 + q, L - 1) * nc;
+            x0[q] = pi[po + a];
+            y0[q] = pi[po + nc + b];
+            fx[q] = pf[po + a];
+            fy[q] = pf[po + nc + b];
+          }
+#pragma unroll
+          for (int q = 0; q < kBatch; ++q) {
+            const LayerDev &Y = I.layers[min(l0 + q, L - 1)];
+            const int N = Y.N, x1 = (x0[q] + 1) & (N - 1), y1 = (y0[q] + 1) & (N - 1);
+            const T *g = phi + Y.off;
+            v00[q] = g[y0[q] * N + x0[q]];
+            v01[q] = g[y0[q] * N + x1];
+            v10[q] = g[y1 * N + x0[q]];
+            v11[q] = g[y1 * N + x1];
+          }
+#pragma unroll
+          for (int q = 0; q < kBatch; ++q)
+            if (l0 + q < L) ps += lerp(fy[q], lerp(fx[q], v00[q], v01[q]), lerp(fx[q], v10[q], v11[q]));
+        }
+        ax.add_prod(tx, ps);
+        ay.add_prod(ty, ps);
+      }
+      const double2 m = block_sum2(ax, ay);
+      if (tid == 0) {
+        T *out = static_cast<T *>(io.out0[it.inst]);
+        out[W.slope_off] = T(m.x / W.S);
+        out[W.slope_off + 1] = T(m.y / W.S);
+      }
+      return;
+    }
     constexpr int U = kFwdChunk / kFwdThreads;
     int at[U][4];
     T fx[U], fy[U], tx[U], ty[U];
@@ -351,6 +381,14 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
         const T p01 = s_psi[w + 1][u], p11 = s_psi[w + 1][u + 1];
         T sx = T(0.5) * (p10 + p11 - p00 - p01);
         T sy = T(0.5) * (p01 + p11 - p00 - p10);
+        if (MODE == 3) {
+          if (u >= 1 && w >= 1) {   // subapertures owned by this tile
+            T *so = static_cast<T *>(io.out0[it.inst]);
+            so[W.slope_off + j] = sx;
+            so[W.slope_off + W.S + j] = sy;
+          }
+          continue;
+        }
         if (MODE == 1) {
           sx = dat[W.slope_off + j] - sx;
           sy = dat[W.slope_off + W.S + j] - sy;
@@ -381,6 +419,7 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
       s_ey[w][u] = ey;
     }
   }
+  if (MODE == 3) return;
   __syncthreads();
   // 3. Gamma^T: each corner gathers its four neighbouring subapertures
   if (lane < kFwdCols) {
@@ -1311,51 +1350,6 @@ __global__ void __launch_bounds__(kThreads) k_update(const InstDev *__restrict__
   }
 }
 
-// ---------------------------------------------------------------- k_slopes
-// Noise-free measurement A phi (eq. atm_tomo): Fried slopes of every valid
-// subaperture, or the two mean slopes of a tip/tilt-only sensor.
-// io.in0: layers; io.out0: slopes.  grid.y = sensor.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_slopes(const InstDev *__restrict__ insts, IoArgs io) {
-  __shared__ InstDev sI;
-  load_inst(&sI, insts);
-  const InstDev &I = sI;
-  const int m = blockIdx.y;
-  const WfsDev W = I.wfs[m];
-  const T *phi = static_cast<const T *>(io.in0[0]);
-  T *out = static_cast<T *>(io.out0[0]);
-  const int nc = W.nc, n = W.n;
-  if (W.kind == kTTOnly) {
-    if (blockIdx.x != 0) return;
-    const T *et = static_cast<const T *>(I.edge_t) + 2 * W.edge_off;
-    const int *eidx = I.edge_idx + W.edge_off;
-    Acc<double> ax, ay;
-    for (int e = threadIdx.x; e < W.n_edge; e += blockDim.x) {
-      const int c = eidx[e];
-      const T ps = trace_corner<T>(I, m, nc, phi, c % nc, c / nc);
-      ax.add_prod(double(et[2 * e]), double(ps));
-      ay.add_prod(double(et[2 * e + 1]), double(ps));
-    }
-    const double2 s = block_sum2(ax, ay);
-    if (threadIdx.x == 0) {
-      out[W.slope_off] = T(s.x / W.S);
-      out[W.slope_off + 1] = T(s.y / W.S);
-    }
-    return;
-  }
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
-  const int a = idx % n, b = idx / n;
-  const int j = I.sub_idx[W.sub_off + idx];
-  if (j < 0) return;
-  const T p00 = trace_corner<T>(I, m, nc, phi, a, b);
-  const T p10 = trace_corner<T>(I, m, nc, phi, a + 1, b);
-  const T p01 = trace_corner<T>(I, m, nc, phi, a, b + 1);
-  const T p11 = trace_corner<T>(I, m, nc, phi, a + 1, b + 1);
-  out[W.slope_off + j] = T(0.5) * (p10 + p11 - p00 - p01);
-  out[W.slope_off + W.S + j] = T(0.5) * (p01 + p11 - p00 - p10);
-}
-
 // --------------------------------------------------------------- k_jacobi
 // Modified Jacobi diagonal (Sec. 5.1), exactly, at plan time and when alpha is retuned:
 //   J_lambda = sum_{m LGS} sigma_m^-2 ||Gamma_m P_m w_lambda||^2 + alpha D_lambda.
@@ -1583,7 +1577,7 @@ cudaError_t allow_type() {
   if (e == cudaSuccess) e = allow_lf<T, 4>();
   if (e == cudaSuccess) e = allow_lf<T, 6>();
   if (e == cudaSuccess) e = allow_lf<T, 8>();
-  const void *fwd[12] = {reinterpret_cast<const void *>(k_forward<T, 0, false, 1>),
+  const void *fwd[14] = {reinterpret_cast<const void *>(k_forward<T, 0, false, 1>),
                          reinterpret_cast<const void *>(k_forward<T, 1, false, 1>),
                          reinterpret_cast<const void *>(k_forward<T, 2, false, 1>),
                          reinterpret_cast<const void *>(k_forward<T, 0, true, 1>),
@@ -1594,8 +1588,10 @@ cudaError_t allow_type() {
                          reinterpret_cast<const void *>(k_forward<T, 2, false, 4>),
                          reinterpret_cast<const void *>(k_forward<T, 0, true, 4>),
                          reinterpret_cast<const void *>(k_forward<T, 1, true, 4>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, true, 4>)};
-  for (int i = 0; i < 12 && e == cudaSuccess; ++i)
+                         reinterpret_cast<const void *>(k_forward<T, 2, true, 4>),
+                         reinterpret_cast<const void *>(k_forward<T, 3, false, 1>),
+                         reinterpret_cast<const void *>(k_forward<T, 3, false, 4>)};
+  for (int i = 0; i < 14 && e == cudaSuccess; ++i)
     e = cudaFuncSetAttribute(fwd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxForwardSmem);
   return e;
 }
@@ -1692,6 +1688,7 @@ cudaError_t fwd_rs(int mode, dim3 g, size_t sm, cudaStream_t s, const InstDev *i
   constexpr int nt = kFwdThreads * 4 / RS;
   if (mode == 0) return launch_ex(k_forward<T, 0, EL, RS>, g, nt, 0, sm, s, insts, items, io);
   if (mode == 1) return launch_ex(k_forward<T, 1, EL, RS>, g, nt, 0, sm, s, insts, items, io);
+  if (mode == 3) return launch_ex(k_forward<T, 3, false, RS>, g, nt, 0, sm, s, insts, items, io);
   return launch_ex(k_forward<T, 2, EL, RS>, g, nt, 0, sm, s, insts, items, io);
 }
 
@@ -1733,14 +1730,6 @@ cudaError_t launch_update(int precision, int flags, const InstDev *insts, int co
                           int n_items, const IoArgs &io, cudaStream_t s) {
   return precision == 0 ? update_t<float>(flags, insts, count, items, n_items, io, s)
                         : update_t<double>(flags, insts, count, items, n_items, io, s);
-}
-
-cudaError_t launch_slopes(int precision, const InstDev *insts, int n_wfs, int max_sub2,
-                          const IoArgs &io, cudaStream_t s) {
-  const dim3 g((max_sub2 + kThreads - 1) / kThreads, n_wfs);
-  if (precision == 0) k_slopes<float><<<g, kThreads, 0, s>>>(insts, io);
-  else k_slopes<double><<<g, kThreads, 0, s>>>(insts, io);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_jacobi(const InstDev *insts, int n_layers, int J, int N_max, const double *prof,

@@ -53,7 +53,7 @@ cudaError_t configure_streamed_kernels();
 cudaError_t configure_gather_kernels();
 
 // Ray-trace, Fried slopes, noise weighting, Gamma^T.  mode 0 operator, 1 residual,
-// 2 data only.  elong: some sensor of the launch has elongated spots.
+// 2 data only, 3 the noise-free measurement of io.in0 into io.out0.  elong: some sensor of the launch has elongated spots.
 cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, const InstDev *insts,
                            const FwdItem *items, int n_items, const IoArgs &io, cudaStream_t s);
 
@@ -62,10 +62,6 @@ cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, c
 cudaError_t launch_update(int precision, int flags, const InstDev *insts, int count, const UpdItem *items,
                           int n_items, const IoArgs &io, cudaStream_t s);
 int update_launches(int n_items);
-
-// Noise-free measurement (single instance).
-cudaError_t launch_slopes(int precision, const InstDev *insts, int n_wfs, int max_sub2,
-                          const IoArgs &io, cudaStream_t s);
 
 // Exact modified Jacobi diagonal (single instance): diag(sum_LGS A~^T C~^-1 A~)
 // + alpha D into jdiag (alpha < 0: the plan's alpha), and its inverse into jinv

@@ -103,7 +103,7 @@ struct tomo_plan {
   tomo::InstDev *d_inst = nullptr;
   double *d_jdiag = nullptr;
   tomo::LaunchSet ls;
-  int nc_max = 0, max_sub2 = 0;
+  int nc_max = 0;
   cudaStream_t cap_stream = nullptr;
   int use_graphs = 1;
   std::vector<tomo::GraphEntry> graphs;
