@@ -865,10 +865,11 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
       continue;
     }
     int tiles = 0;
-    for (int b0 = 0; b0 < d.nc; b0 += kFwdRows)
+    const int fr = fwd_rows(P->precision);
+    for (int b0 = 0; b0 < d.nc; b0 += fr)
       for (int a0 = 0; a0 < d.nc; a0 += kFwdCols) {
         bool any = false;
-        for (int b = b0; b < std::min(d.nc, b0 + kFwdRows) && !any; ++b)
+        for (int b = b0; b < std::min(d.nc, b0 + fr) && !any; ++b)
           for (int a = a0; a < std::min(d.nc, a0 + kFwdCols) && !any; ++a)
             any = P->active[d.act_off + b * d.nc + a] != 0;
         if (!any) continue;

@@ -87,7 +87,7 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 // formed once for the corner rows above and below it: RS + 1 node rows are read
 // per layer instead of 2 RS, all requested before any is used.
 //
-// RS = 4 (kFwdThreads threads) for big launches, RS = 1 (four times the
+// RS = kFwdStrip (4, FP64 2: kFwdThreads threads) for big launches, RS = 1 (more
 // warps, no reuse, less work in a chain) for small ones.  The steps that feed
 // the tile's partial sums (the slopes and the tip/tilt-only chunks) keep a
 // fixed kFwdThreads-thread mapping, so the partials, and every result, are
@@ -98,7 +98,14 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 // layer (GB300, cold launch): 16 E-ELT systems 49.2 -> 33 us, 64 uneven systems
 // 50.9 -> 34 us, the 100 m system 54.0 -> 46 us.
 constexpr size_t kFwdSmallSmem = 64 * 1024;
-constexpr int kFwdLanes = kFwdCols + 2, kFwdPsi = kFwdRows + 2;
+constexpr int kFwdLanes = kFwdCols + 2;
+template <typename T>
+constexpr int kFwdRows = fwd_rows(sizeof(T) == 8);
+template <typename T>
+constexpr int kFwdPsi = kFwdRows<T> + 2;
+// rows per warp of big launches (kFwdThreads threads)
+template <typename T>
+constexpr int kFwdStrip = kFwdPsi<T> * 32 / kFwdThreads;
 
 // Shared memory of the staged corner tables of L layers: per layer the grid
 // side and offset, the columns' node index and fraction, and per corner row
@@ -111,7 +118,7 @@ struct FwdRow {
 };
 template <typename T>
 __host__ __device__ constexpr size_t fwd_table_bytes(int L) {
-  return L * (kFwdPsi * sizeof(FwdRow<T>) + kFwdLanes * sizeof(T) + (kFwdLanes + 2) * sizeof(int)) + 16;
+  return L * (kFwdPsi<T> * sizeof(FwdRow<T>) + kFwdLanes * sizeof(T) + (kFwdLanes + 2) * sizeof(int)) + 16;
 }
 
 // (1 - f) a + f b, rounded the same way wherever it is used.
@@ -147,7 +154,7 @@ __device__ __forceinline__ void trace_strip(const T *__restrict__ phi, int L, in
       int last = 0;
 #pragma unroll
       for (int j = 0; j < RS; ++j) {
-        const FwdRow<T> row = s_row[l * kFwdPsi + w + j];
+        const FwdRow<T> row = s_row[l * kFwdPsi<T> + w + j];
         const int rj = row.y0 << lgN, r1 = (rj + N) & mask;
         r0[q][j] = rj;
         fy[q][j] = row.f;
@@ -188,12 +195,12 @@ __device__ __forceinline__ void trace_strip(const T *__restrict__ phi, int L, in
 }
 
 template <typename T, int MODE, bool EL, int RS>
-__global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
+__global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T) == 4 ? 8 : 4))
     k_forward(const InstDev *__restrict__ insts, const FwdItem *__restrict__ items, IoArgs io) {
   extern __shared__ __align__(16) unsigned char fsm[];
-  __shared__ T s_psi[kFwdPsi][kFwdLanes + 1];
-  __shared__ T s_ex[kFwdRows + 1][kFwdLanes];
-  __shared__ T s_ey[kFwdRows + 1][kFwdLanes];
+  __shared__ T s_psi[kFwdPsi<T>][kFwdLanes + 1];
+  __shared__ T s_ex[kFwdRows<T> + 1][kFwdLanes];
+  __shared__ T s_ey[kFwdRows<T> + 1][kFwdLanes];
   pdl_trigger();
   const FwdItem it = items[blockIdx.x];
   if (io.active && !io.active[it.inst]) return;
@@ -300,7 +307,7 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
 
   // stage this tile's corner->node tables for every layer (constant data)
   FwdRow<T> *s_row = reinterpret_cast<FwdRow<T> *>(fsm);
-  T *s_fx = reinterpret_cast<T *>(s_row + L * kFwdPsi);
+  T *s_fx = reinterpret_cast<T *>(s_row + L * kFwdPsi<T>);
   int *s_x0 = reinterpret_cast<int *>(s_fx + L * kFwdLanes);
   int *s_N = s_x0 + L * kFwdLanes;
   int *s_off = s_N + L;
@@ -312,8 +319,8 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
       cp_async_elem(s_x0 + idx, pi + a);
       cp_async_elem(s_fx + idx, pf + a);
     }
-    for (int idx = tid; idx < L * kFwdPsi; idx += nt) {
-      const int l = idx / kFwdPsi, w = idx - l * kFwdPsi;
+    for (int idx = tid; idx < L * kFwdPsi<T>; idx += nt) {
+      const int l = idx / kFwdPsi<T>, w = idx - l * kFwdPsi<T>;
       const int b = 2 * l * nc + nc + min(max(b0 - 1 + w, 0), nc - 1);
       cp_async_elem(&s_row[idx].y0, pi + b);
       cp_async_elem(&s_row[idx].f, pf + b);
@@ -328,12 +335,12 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
   const int *sidx = I.sub_idx + W.sub_off;
   const int lane = tid & 31, warp = tid >> 5;
   // the slope indices of step 2 (constant: before the dependency wait)
-  constexpr int kSubRounds = (kFwdRows + kFwdThreads / 32) / (kFwdThreads / 32);
+  constexpr int kSubRounds = (kFwdRows<T> + kFwdThreads / 32) / (kFwdThreads / 32);
   int sj[kSubRounds];
 #pragma unroll
   for (int q = 0; q < kSubRounds; ++q) {
     const int w = warp + q * (kFwdThreads / 32), a = a0 - 1 + lane, b = b0 - 1 + w;
-    sj[q] = tid < kFwdThreads && lane <= kFwdCols && w <= kFwdRows && a >= 0 && b >= 0 && a < n && b < n
+    sj[q] = tid < kFwdThreads && lane <= kFwdCols && w <= kFwdRows<T> && a >= 0 && b >= 0 && a < n && b < n
                 ? sidx[b * n + a]
                 : -1;
   }
@@ -374,7 +381,7 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
 #pragma unroll
     for (int q = 0; q < kSubRounds; ++q) {
       const int w = warp + q * (kFwdThreads / 32), b = b0 - 1 + w, j = sj[q];
-      if (w > kFwdRows) break;
+      if (w > kFwdRows<T>) break;
       T ex = T(0), ey = T(0);
       if (j >= 0) {
         const T p00 = s_psi[w][u], p10 = s_psi[w][u + 1];
@@ -424,7 +431,7 @@ __global__ void __launch_bounds__(kFwdThreads * 4 / RS, RS == 1 ? 2 : 8)
   // 3. Gamma^T: each corner gathers its four neighbouring subapertures
   if (lane < kFwdCols) {
     const int u = lane, a = a0 + u;
-    for (int w = warp; w < kFwdRows; w += nt >> 5) {
+    for (int w = warp; w < kFwdRows<T>; w += nt >> 5) {
       const int b = b0 + w;
       if (a < nc && b < nc) {
         const T val = T(0.5) * (s_ex[w + 1][u] + s_ex[w][u] - s_ex[w + 1][u + 1] - s_ex[w][u + 1]) +
@@ -1583,14 +1590,14 @@ cudaError_t allow_type() {
                          reinterpret_cast<const void *>(k_forward<T, 0, true, 1>),
                          reinterpret_cast<const void *>(k_forward<T, 1, true, 1>),
                          reinterpret_cast<const void *>(k_forward<T, 2, true, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 0, false, 4>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, false, 4>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, false, 4>),
-                         reinterpret_cast<const void *>(k_forward<T, 0, true, 4>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, true, 4>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, true, 4>),
+                         reinterpret_cast<const void *>(k_forward<T, 0, false, kFwdStrip<T>>),
+                         reinterpret_cast<const void *>(k_forward<T, 1, false, kFwdStrip<T>>),
+                         reinterpret_cast<const void *>(k_forward<T, 2, false, kFwdStrip<T>>),
+                         reinterpret_cast<const void *>(k_forward<T, 0, true, kFwdStrip<T>>),
+                         reinterpret_cast<const void *>(k_forward<T, 1, true, kFwdStrip<T>>),
+                         reinterpret_cast<const void *>(k_forward<T, 2, true, kFwdStrip<T>>),
                          reinterpret_cast<const void *>(k_forward<T, 3, false, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 3, false, 4>)};
+                         reinterpret_cast<const void *>(k_forward<T, 3, false, kFwdStrip<T>>)};
   for (int i = 0; i < 14 && e == cudaSuccess; ++i)
     e = cudaFuncSetAttribute(fwd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxForwardSmem);
   return e;
@@ -1685,7 +1692,7 @@ cudaError_t launch_analysis(int precision, int src, int epi, int lf, int flags, 
 template <typename T, bool EL, int RS>
 cudaError_t fwd_rs(int mode, dim3 g, size_t sm, cudaStream_t s, const InstDev *insts, const FwdItem *items,
                    const IoArgs &io) {
-  constexpr int nt = kFwdThreads * 4 / RS;
+  constexpr int nt = 32 * kFwdPsi<T> / RS;
   if (mode == 0) return launch_ex(k_forward<T, 0, EL, RS>, g, nt, 0, sm, s, insts, items, io);
   if (mode == 1) return launch_ex(k_forward<T, 1, EL, RS>, g, nt, 0, sm, s, insts, items, io);
   if (mode == 3) return launch_ex(k_forward<T, 3, false, RS>, g, nt, 0, sm, s, insts, items, io);
@@ -1696,7 +1703,7 @@ template <typename T, bool EL>
 cudaError_t fwd_t(int mode, dim3 g, size_t sm, cudaStream_t s, const InstDev *insts, const FwdItem *items,
                   const IoArgs &io) {
   return g.x <= kFwdSmallLaunch ? fwd_rs<T, EL, 1>(mode, g, sm, s, insts, items, io)
-                                : fwd_rs<T, EL, 4>(mode, g, sm, s, insts, items, io);
+                                : fwd_rs<T, EL, kFwdStrip<T>>(mode, g, sm, s, insts, items, io);
 }
 
 cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, const InstDev *insts,
