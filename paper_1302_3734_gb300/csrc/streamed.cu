@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(kDwtThreads) k_dwt_pass(const InstDev *__restr
 }
 
 // The coarse analysis levels ks..J of one layer in one CTA: the block of side
-// N >> (ks - 1) from the scratch (or, ks = 1, the layer grid); every output emitted.
+// N >> (ks - 1) from the scratch (or, ks = 1, the layer grid); every output emitted,
+// its epilogue input from shared memory, where it arrives with the block.
 template <typename T, int SRC, int EPI, int LF>
 __global__ void __launch_bounds__(kPassThreads) k_dwt_coarse(const InstDev *__restrict__ insts,
                                                              const PassItem *__restrict__ items, IoArgs io,
@@ -228,10 +229,12 @@ __global__ void __launch_bounds__(kPassThreads) k_dwt_coarse(const InstDev *__re
   load_inst(&sI, insts + it.inst);
   const InstDev &I = sI;
   const LayerDev &L = I.layers[it.layer];
-  const int J = I.J, tid = threadIdx.x, nt = blockDim.x, ks = L.ks;
+  const int J = I.J, tid = threadIdx.x, nt = blockDim.x, ks = L.ks, N = L.N;
   int lgM = L.log2N - (ks - 1), M = 1 << lgM;
   T *A = reinterpret_cast<T *>(smem_raw);
   T *B = A + M * M;
+  T *E = B + M * M;   // the epilogue's p (or x) of the block
+  const int lgM0 = lgM;
   if (tid <= J) s_dal[tid] = T(L.dalpha[tid]);
   Filt<T, LF> f;
   f.load(I);
@@ -242,6 +245,12 @@ __global__ void __launch_bounds__(kPassThreads) k_dwt_coarse(const InstDev *__re
   __syncthreads();
   pdl_wait();
   stage_rows_async<T>(A, src, M, 0, M, M, M - 1);
+  const bool staged = EPI == kEpiOp || (EPI == kEpiResid && emit.warm);
+  if (staged) {
+    stage_rows_async<T>(E, (EPI == kEpiOp ? emit.P : emit.X) + L.off, N, 0, M, M, M - 1);
+    emit.cache = E;
+  }
+  auto slot = [&](int row, int col) { return staged ? (row << lgM0) + col : -1; };
   cp_async_wait_all();
   __syncthreads();
   for (int k = ks; k <= J; ++k, M >>= 1, --lgM) {
@@ -265,8 +274,8 @@ __global__ void __launch_bounds__(kPassThreads) k_dwt_coarse(const InstDev *__re
           }
           lo[u] = l;
           hi[u] = h;
-          if (!(x < H && k < J)) fa[u] = emit.fetch(i, x, -1);
-          fb[u] = emit.fetch(H + i, x, -1);
+          if (!(x < H && k < J)) fa[u] = emit.fetch(i, x, slot(i, x));
+          fb[u] = emit.fetch(H + i, x, slot(H + i, x));
         }
       }
 #pragma unroll
@@ -352,8 +361,9 @@ struct SynthCoef {
   }
 };
 
-// Coefficients (and low-low values) staged per thread at once by the synthesis kernels.
-constexpr int kCoefU = 4;
+// Coefficients (and low-low values) staged per thread at once by the synthesis kernels; the
+// coarse kernel's share of a 64 x 64 block.
+constexpr int kCoefU = 4, kCoarseCoefU = 8;
 
 // 16 bytes of T: the unit of the vector loads of the streamed synthesis pass.
 template <typename T>
@@ -406,22 +416,27 @@ __global__ void __launch_bounds__(kPassThreads) k_idwt_coarse(const InstDev *__r
   Filt<T, LF> f;
   f.load(I);
   pdl_wait();
-  const T beta = SRC == 1 ? streamed_beta<T>(I, flags >> kIterShift, true) : T(0);
-  const SynthCoef<T, SRC> coef = synth_coef<T, SRC>(I, io, it.inst, flags, beta);
-  for (int idx0 = tid; idx0 < M0 * M0; idx0 += kCoefU * nt) {
-    typename SynthCoef<T, SRC>::Raw raw[kCoefU];
+  SynthCoef<T, SRC> coef = synth_coef<T, SRC>(I, io, it.inst, flags, T(0));
+  auto at = [&](int idx) { return static_cast<size_t>(L.off) + static_cast<size_t>(idx >> lgM0) * N + (idx & (M0 - 1)); };
+  // the first coefficients of each thread are requested before beta is formed
+  typename SynthCoef<T, SRC>::Raw raw[kCoarseCoefU];
 #pragma unroll
-    for (int u = 0; u < kCoefU; ++u) {
-      const int idx = idx0 + u * nt;
-      if (idx < M0 * M0)
-        raw[u] = coef.load(static_cast<size_t>(L.off) + static_cast<size_t>(idx >> lgM0) * N + (idx & (M0 - 1)));
-    }
+  for (int u = 0; u < kCoarseCoefU; ++u)
+    if (tid + u * nt < M0 * M0) raw[u] = coef.load(at(tid + u * nt));
+  if (SRC == 1) coef.beta = streamed_beta<T>(I, flags >> kIterShift, true);
 #pragma unroll
-    for (int u = 0; u < kCoefU; ++u) {
+  for (int u = 0; u < kCoarseCoefU; ++u) {
+    const int idx = tid + u * nt;
+    if (idx < M0 * M0) Cf[idx] = coef.value(raw[u], at(idx), true);
+  }
+  for (int idx0 = tid + kCoarseCoefU * nt; idx0 < M0 * M0; idx0 += kCoarseCoefU * nt) {
+#pragma unroll
+    for (int u = 0; u < kCoarseCoefU; ++u)
+      if (idx0 + u * nt < M0 * M0) raw[u] = coef.load(at(idx0 + u * nt));
+#pragma unroll
+    for (int u = 0; u < kCoarseCoefU; ++u) {
       const int idx = idx0 + u * nt;
-      if (idx < M0 * M0)
-        Cf[idx] = coef.value(raw[u], static_cast<size_t>(L.off) + static_cast<size_t>(idx >> lgM0) * N + (idx & (M0 - 1)),
-                             true);
+      if (idx < M0 * M0) Cf[idx] = coef.value(raw[u], at(idx), true);
     }
   }
   __syncthreads();
