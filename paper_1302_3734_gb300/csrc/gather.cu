@@ -33,7 +33,7 @@ namespace tomo {
 // each and every corner row summed for every band (GB300, cold launch): 16
 // E-ELT systems 49.2 -> 35.6 us, 64 uneven systems 82.9 -> 63 us, the 100 m
 // system 82.2 -> 61.1 us.
-constexpr int kWalk = 4;
+constexpr int kWalk = 2;
 
 template <typename T, int KT>
 __device__ __forceinline__ T col_sum(const T *wx, const T *v) {
