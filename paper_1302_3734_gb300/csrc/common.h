@@ -25,7 +25,9 @@ constexpr int kFwdSmallLaunch = 608;   // forward CTAs up to which a launch is s
 constexpr int kAnalysisThreads = 512;  // threads per CTA of the gather + analysis kernel when two fit an SM
 constexpr int kAnalysisThreadsMax = 1024;  // ... when its shared memory leaves room for one
 constexpr int kSynthThreads = 512;     // threads per CTA of the synthesis kernel (at most)
-constexpr int kGatherThreads = 384;    // threads per CTA of the separate gather kernel
+// Threads per CTA of the separate gather kernel (solve loops of 16 E-ELT / 64 uneven / 100 m
+// systems, us: 512: 1181 / 2943 / 2763, 384: 1167 / 2872 / 2785, 256: 1239 / 2881 / 2852).
+constexpr int kGatherThreads = 384;
 constexpr int kMaxGatherSensors = 64;  // dense sensors the separate gather kernel lists
 constexpr int kUpdChunk = 1024;    // coefficients per pass of a vector-update CTA
 constexpr int kUpdMaxBlocks = 608; // update CTAs per instance at most (four per SM of 152 SMs)

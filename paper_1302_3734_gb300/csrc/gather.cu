@@ -31,8 +31,9 @@ namespace tomo {
 // Bound by latency (barriers, the stages' copies) at two CTAs per SM.  Against
 // one pass for the column sums and one for the nodes, with a barrier after
 // each and every corner row summed for every band (GB300, cold launch): 16
-// E-ELT systems 49.2 -> 35.6 us, 64 uneven systems 82.9 -> 63 us, the 100 m
-// system 82.2 -> 61.1 us.
+// E-ELT systems 49.2 -> 33.5 us, 64 uneven systems 82.9 -> 54.4 us, the 100 m
+// system 82.2 -> 55.4 us.
+// (Four rows took 16 E-ELT systems 2% longer: one skipped corner row sends the batch to whole windows.)
 constexpr int kWalk = 2;
 
 template <typename T, int KT>

@@ -95,8 +95,8 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 //
 // Bound by instruction issue and L1 in big launches, by latency in small ones.
 // Against one corner per thread on 18 x 18 corners, four loads per corner and
-// layer (GB300, cold launch): 16 E-ELT systems 49.2 -> 33 us, 64 uneven systems
-// 50.9 -> 34 us, the 100 m system 54.0 -> 46 us.
+// layer (GB300, cold launch): 16 E-ELT systems 49.2 -> 29 us, 64 uneven systems
+// 50.9 -> 29 us, the 100 m system 54.0 -> 43 us.
 constexpr size_t kFwdSmallSmem = 64 * 1024;
 constexpr int kFwdLanes = kFwdCols + 2;
 template <typename T>

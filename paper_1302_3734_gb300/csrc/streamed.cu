@@ -83,9 +83,12 @@ constexpr int kEmitU = 4;
 // input rows, their row transforms from the lane's window of LF + 2 inputs
 // (16-byte loads; the neighbours' overlap hits the L1), then the column sums
 // over the last LF row transforms, which stay in registers.  No shared memory
-// and no barrier before the partial sums.  (Staging the tile's rows and their
-// row transforms in shared memory for two barrier-separated passes, one output
-// column per thread, took about four times the instructions.)
+// and no barrier before the partial sums.  Bound by the epilogue's traffic (p in,
+// q out) and the latency of the row loads.  Against staging the tile's rows and
+// their row transforms in shared memory for two barrier-separated passes, one
+// output column per thread (GB300, cold launch): finest pass of the 100 m system
+// 51.2 -> 32 us, of 64 uneven systems 71.6 -> 35 us, of 16 E-ELT systems 25.8 ->
+// 14 us.
 template <typename T>
 struct alignas(16) Quad {
   T v[4];
@@ -215,7 +218,8 @@ __global__ void __launch_bounds__(kDwtThreads) k_dwt_pass(const InstDev *__restr
 
 // The coarse analysis levels ks..J of one layer in one CTA: the block of side
 // N >> (ks - 1) from the scratch (or, ks = 1, the layer grid); every output emitted,
-// its epilogue input from shared memory, where it arrives with the block.
+// its epilogue input from shared memory, where it arrives with the block (GB300,
+// cold: 16 E-ELT systems 11.2 us with the inputs read level by level, 9.6 so).
 template <typename T, int SRC, int EPI, int LF>
 __global__ void __launch_bounds__(kPassThreads) k_dwt_coarse(const InstDev *__restrict__ insts,
                                                              const PassItem *__restrict__ items, IoArgs io,
@@ -418,7 +422,8 @@ __global__ void __launch_bounds__(kPassThreads) k_idwt_coarse(const InstDev *__r
   pdl_wait();
   SynthCoef<T, SRC> coef = synth_coef<T, SRC>(I, io, it.inst, flags, T(0));
   auto at = [&](int idx) { return static_cast<size_t>(L.off) + static_cast<size_t>(idx >> lgM0) * N + (idx & (M0 - 1)); };
-  // the first coefficients of each thread are requested before beta is formed
+  // the first coefficients of each thread are requested before beta is formed (GB300, cold: 16
+  // E-ELT systems 14.2 -> 10.3 us)
   typename SynthCoef<T, SRC>::Raw raw[kCoarseCoefU];
 #pragma unroll
   for (int u = 0; u < kCoarseCoefU; ++u)
@@ -502,7 +507,12 @@ __global__ void __launch_bounds__(kPassThreads) k_idwt_coarse(const InstDev *__r
 // syntheses of the low-y and the high-y row from 16-byte windows, and the column
 // synthesis over the last LF/2 half-rows, whose row syntheses stay in registers.
 // One barrier; a strip repeats the row syntheses of HL half-rows, so a tile has
-// at most four strips.
+// at most four strips.  Bound by the coefficients' loads (DRAM and their latency
+// at four or five CTAs per SM).  Against writing the row syntheses back to shared
+// memory for a second pass (GB300, cold launch): 64 uneven systems 57.7 -> 39 us,
+// 16 E-ELT systems 20.1 -> 14 us, the 100 m system's finest pass 45.4 -> 38 us.
+// (Without the staging, each thread reading its window from global memory, the
+// halo columns are updated twice: 57 us there.)
 template <typename T, int SRC, int LF>
 __global__ void __launch_bounds__(kIdwtThreads) k_idwt_pass(const InstDev *__restrict__ insts,
                                                             const PassItem *__restrict__ items, IoArgs io,
