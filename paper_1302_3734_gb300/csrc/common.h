@@ -34,7 +34,7 @@ constexpr int kUpdMaxBlocks = 608; // update CTAs per instance at most (four per
 constexpr int kUpdAlphaBlocks = kUpdMaxBlocks;   // update CTAs of a launch above which k_alpha forms alpha first
 constexpr int kMaxTapsNode = 4;    // corners per axis whose bilinear taps reach one node
 constexpr int kPassRows = 8;       // half-rows of a level one CTA of a streamed transform pass covers
-constexpr int kPassThreads = 512;  // threads per CTA of the streamed transform kernels
+constexpr int kPassThreads = 512;  // threads per CTA of the streamed coarse kernels
 constexpr int kDwtThreads = 128;   // threads per CTA of a streamed analysis pass (kPassRows half-rows)
 constexpr int kIdwtThreads = 128;  // ... and of a streamed synthesis pass
 constexpr int kCoarseMax = 64;     // block side up to which one CTA finishes a layer's transform
@@ -307,9 +307,9 @@ struct StreamSet {
   size_t smem_pass = 0, smem_coarse = 0;
 };
 
-// Shared memory of a streamed pass at block side M (elements of T): the analysis
-// stages 2 kPassRows + LF - 2 input rows and their row transforms; the synthesis
-// 2 (kPassRows + LF/2 - 1) coefficient rows and their row syntheses.
+// Size of a streamed pass at block side M (elements of T), the bound up to which
+// layers are accepted: the synthesis stages half of it, 2 (kPassRows + LF/2 - 1)
+// coefficient rows; the analysis uses no shared memory.
 TOMO_HD inline int pass_smem_elems(int M, int LF) {
   const int a = 2 * (2 * kPassRows + LF - 2) * M;
   const int s = 4 * (kPassRows + LF / 2 - 1) * M;
