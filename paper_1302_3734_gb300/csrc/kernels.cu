@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
     if constexpr (MODE == 3) {
       if (it.tile != 0) return;
       pdl_wait();
-      Acc<T> ax, ay;
+      // (the measurement's sums are FP64 in FP32 plans too: one CTA per sensor, a term or two per thread)
+      Acc<double> ax, ay;
       constexpr int kBatch = 5;   // layers whose loads a thread issues together
       for (int e = tid; e < W.n_edge; e += nt) {
         const int c = I.edge_idx[W.edge_off + e], a = c % nc, b = c / nc;
@@ -254,8 +255,8 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
           for (int q = 0; q < kBatch; ++q)
             if (l0 + q < L) ps += lerp(fy[q], lerp(fx[q], v00[q], v01[q]), lerp(fx[q], v10[q], v11[q]));
         }
-        ax.add_prod(tx, ps);
-        ay.add_prod(ty, ps);
+        ax.add_prod(double(tx), double(ps));
+        ay.add_prod(double(ty), double(ps));
       }
       const double2 m = block_sum2(ax, ay);
       if (tid == 0) {
