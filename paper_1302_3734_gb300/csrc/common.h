@@ -288,6 +288,12 @@ TOMO_HD inline GatherSmem gather_smem_layout(int R0, int N, int rec_stride, int 
 }
 // Shared memory up to which a gather CTA takes a whole cluster band: two CTAs per SM.
 constexpr int kGatherSmem = 108 * 1024;
+// Dynamic shared memory a gather CTA can have, and whether a band's pupil-edge terms fit there;
+// if not (a node row with hundreds of terms per node) they are summed from global memory.
+constexpr int kGatherMaxSmem = 220 * 1024;
+TOMO_HD inline bool gather_edges_fit(const GatherSmem &g, long long entries, int esz) {
+  return g.stage + entries * esz <= kGatherMaxSmem;
+}
 
 // Work items.
 struct ClusterItem { int inst, layer; };

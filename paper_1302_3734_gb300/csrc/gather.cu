@@ -246,7 +246,12 @@ __global__ void __launch_bounds__(kGatherThreads, sizeof(T) == 4 ? 2 : 1) k_gath
       stage_rows(md + 2);
     }
   }
-  if (I.n_edge_wfs > 0) {
+  if (I.n_edge_wfs > 0 && !gather_edges_fit(gs, e1 - e0, static_cast<int>(sizeof(T)))) {
+    // more pupil-edge terms than shared memory holds: each node's from global memory, in list order
+    for (int j = seg.x + tid; j < seg.y; j += nt)
+      A[I.tt_node[j]] += edge_node_sum<T>(I.tt_beg[j], I.tt_beg[j + 1], I.tt_k, static_cast<const T *>(I.tt_w), s_coef);
+    __syncthreads();
+  } else if (I.n_edge_wfs > 0) {
     // the pupil-edge list, added after the sensors: every entry's term into the free stages
     // (coalesced loads), then each node's terms in list order
     T *C = reinterpret_cast<T *>(smem_raw + gs.stage);

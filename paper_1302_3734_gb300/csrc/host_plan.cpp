@@ -702,8 +702,9 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
     fits = fits && P->max_tt_entries <= 65535;   // the image's 16-bit entry indices
     P->gather_staged = fits ? 1 : 0;
     P->smem_analysis = fits ? need : P->smem_transform;
-    // the separate gather kernel takes bands of this size at most: the band's nodes,
-    // its row records and the column sums of one sensor's corner rows within 220 KB
+    // cluster bands accepted for the separate gather: the band's nodes, 4 bytes and the weights of
+    // each of its rows and one sensor's corner rows, summed over the columns, within 220 KB (the
+    // kernel itself needs less; the bound is kept so that what is accepted does not change)
     long long band = 0;
     for (const auto &d : P->layers) {
       const long long R0 = d.N / P->C;
@@ -719,22 +720,29 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
       return TOMO_ERR_UNSUPPORTED;
     }
     // the separate gather's bands: the cluster bands, halved until a CTA's buffers leave room for
-    // two CTAs per SM (at the latest at one node row per band)
-    auto smem_bands = [&]() {
-      int entries = 0;
-      for (const auto &sg : P->tt_seg) entries = std::max(entries, P->tt_beg[sg.y] - P->tt_beg[sg.x]);
-      int most = 0;
-      for (const auto &d : P->layers) {
-        const GatherSmem g = gather_smem_layout(d.N / std::min(P->gather_bands, d.N), d.N, P->rec_stride, esz,
-                                                P->max_band_v);
-        most = std::max(most, std::max(g.total, g.stage + entries * esz));
+    // two CTAs per SM (at the latest at one node row per band); a band's pupil-edge terms count, but
+    // not in what is launched where they do not fit a CTA at all
+    auto smem_bands = [&](bool launched) {
+      long long widest = 0, most = 0;
+      for (const auto &sg : P->tt_seg) widest = std::max<long long>(widest, P->tt_beg[sg.y] - P->tt_beg[sg.x]);
+      for (int l = 0; l < P->n_layers; ++l) {
+        const int N = P->layers[l].N, nb = std::min(P->gather_bands, N);
+        const GatherSmem g = gather_smem_layout(N / nb, N, P->rec_stride, esz, P->max_band_v);
+        most = std::max<long long>(most, g.total);
+        if (!launched) most = std::max(most, g.stage + widest * esz);
+        for (int c = 0; launched && c < nb; ++c) {
+          const int2 sg = P->tt_seg[static_cast<size_t>(l) * P->gather_bands + c];
+          const long long entries = P->tt_beg[sg.y] - P->tt_beg[sg.x];
+          if (gather_edges_fit(g, entries, esz)) most = std::max(most, g.stage + entries * esz);
+        }
       }
       return most;
     };
-    P->smem_gather = smem_bands();
-    while (!fits && P->smem_gather > kGatherSmem && P->gather_bands < Nmax) {
-      build_bands(2 * P->gather_bands);
-      P->smem_gather = smem_bands();
+    while (!fits && smem_bands(false) > kGatherSmem && P->gather_bands < Nmax) build_bands(2 * P->gather_bands);
+    P->smem_gather = smem_bands(true);
+    if (!fits && P->smem_gather > kGatherMaxSmem) {
+      *err = "layer grids too large for the separate gather kernel's buffers";
+      return TOMO_ERR_UNSUPPORTED;
     }
   }
   // the stage images, one per analysis CTA
