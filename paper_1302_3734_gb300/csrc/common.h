@@ -206,11 +206,17 @@ TOMO_HD inline int tile_partials(const WfsDev &d) { return (d.elong && d.kind ==
 // transform alone: a level over the cluster costs two barriers and a round trip
 // to the neighbours (about 2 us), one of a 32 x 32 block in one CTA less than
 // half of that.  Against S = C (GB300, 10 iterations): one E-ELT frame 416 ->
-// 407 us, one 8 m frame 222 -> 209 us.  At most 32 and N / 2, at least C (a row per CTA), and the
-// block and its row transforms fit one of the two row buffers.
-TOMO_HD inline int transform_coarse_side(int N, int C) {
+// 407 us, one 8 m frame 222 -> 209 us.  At most N / 2, at least C (a row per CTA), and the
+// block and its row transforms fit one of the two row buffers.  At most 32, but 16
+//  - in FP64, where one SM's FP64 pipe takes longer over a 32 x 32 block than the cluster (normal
+//    operator, 128 x 128 layers, us with 32 and 16: 5 layers db4 93.7 and 76.9, 7 layers db2 94 and 84);
+//  - where a block of 32 would hold one level or none: its gather and two barriers then replace
+//    as many (128 x 128 layers, 3 levels, S = 32 and 16: 5 layers db4 25.3 and 24.6 us, 3 layers db3
+//    23.9 and 22.6 us).
+TOMO_HD inline int transform_coarse_side(int N, int C, int J, int precision) {
+  const int most = precision || (N >> (J - 1)) >= 32 ? 16 : 32;
   int s = C;
-  while (2 * s <= 32 && 2 * s <= N / 2 && 2 * (2 * s) * (2 * s) <= (N / C + kMaxTaps) * N) s *= 2;
+  while (2 * s <= most && 2 * s <= N / 2 && 2 * (2 * s) * (2 * s) <= (N / C + kMaxTaps) * N) s *= 2;
   return s;
 }
 

@@ -208,7 +208,7 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
     long long need = 0;
     cluster_fits = true;
     for (auto &d : P->layers) {
-      d.coarse = wide ? transform_coarse_side(d.N, P->C) : P->C;
+      d.coarse = wide ? transform_coarse_side(d.N, P->C, J, P->precision) : P->C;
       const long long base = transform_cache_offset(d.N, P->C, d.coarse);
       int kc = 1;
       while (kc <= J && (base + transform_cache_size(d.N, P->C, d.coarse, J, kc)) * esz > budget) ++kc;

@@ -1,14 +1,7 @@
-"""Systems at the limits of the separate gather kernel, and their host-plan sizes."""
-import ctypes
-import math
-import os
-import subprocess
-
+"""Systems at the limits of the separate gather kernel."""
 import numpy as np
 
 from synth import configs
-
-HERE = os.path.dirname(os.path.abspath(__file__))
 
 
 def many_edge_terms(n_tt):
@@ -28,18 +21,3 @@ def many_edge_terms(n_tt):
                                     theta=tuple(rng.uniform(0.25, 0.75, 2) * dx / 1000.0)) for k in range(n_tt)]
     g["D_tel"] = n * 2 * dx
     return g
-
-
-def host_plan_sizes(geom, cluster_size, transforms, folder):
-    """(bands, shared memory, terms of the largest band) of the separate gather, from the host plan alone."""
-    from paper_1302_3734_gb300 import build, geometry_struct
-    lib = os.path.join(str(folder), "libhostplan.so")
-    if not os.path.exists(lib):
-        subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", f"-I{build.INCLUDE}", f"-I{build.CSRC}",
-                        f"-I{os.path.join(build._cuda_home(), 'include')}", os.path.join(HERE, "host_plan_probe.cpp"),
-                        os.path.join(build.CSRC, "host_plan.cpp"), "-o", lib], check=True)
-    g, keep = geometry_struct(geom)
-    out = (ctypes.c_longlong * 3)()
-    st = ctypes.CDLL(lib).host_plan_gather(ctypes.byref(g), cluster_size, transforms, out)
-    assert st == 0, st
-    return list(out)

@@ -18,3 +18,13 @@ extern "C" int host_plan_gather(const tomo_geometry *g, int cluster_size, int tr
   }
   return TOMO_OK;
 }
+
+// out[0..n_layers): side of the block that one CTA of a layer's cluster finishes.
+extern "C" int host_plan_coarse(const tomo_geometry *g, int cluster_size, int transforms, long long *out) {
+  tomo::HostPlan P;
+  std::string err;
+  const int st = tomo::build_host_plan(g, &P, &err, cluster_size, transforms);
+  if (st != TOMO_OK) return st;
+  for (size_t l = 0; l < P.layers.size(); ++l) out[l] = P.layers[l].coarse;
+  return TOMO_OK;
+}

@@ -6,7 +6,8 @@ relative L2 below 1e-11 as for the other FP64 operator checks.
 import numpy as np
 import pytest
 
-from gather_systems import host_plan_sizes, many_edge_terms
+from gather_systems import many_edge_terms
+from host_plan import gather_sizes
 from oracle import Tomography
 
 pytestmark = pytest.mark.gpu
@@ -19,7 +20,7 @@ def test_rhs_with_bands_of_one_row(n_tt, tmp_path):
     from paper_1302_3734_gb300.binding import Plan
     build.build()
     g = many_edge_terms(n_tt)
-    assert host_plan_sizes(g, 64, 2, tmp_path)[0] == max(l["N"] for l in g["layers"]) > min(l["N"] for l in g["layers"])
+    assert gather_sizes(g, 64, 2, tmp_path)[0] == max(l["N"] for l in g["layers"]) > min(l["N"] for l in g["layers"])
     plan = Plan(g, cluster_size=64, transforms=2)
     s = np.random.default_rng(n_tt).standard_normal(plan.n_slopes)
     out = torch.empty(plan.n, dtype=torch.float64, device="cuda")

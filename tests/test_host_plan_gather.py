@@ -1,11 +1,9 @@
 """Shared memory of the separate gather, from the host plan alone: a plan that is accepted
 can be launched (220 KB a CTA), also where one node row has more pupil-edge terms than fit."""
-import math
-
 import pytest
 
-from gather_systems import host_plan_sizes, many_edge_terms
-from synth import configs
+from gather_systems import many_edge_terms
+from host_plan import gather_sizes
 
 LIMIT = 220 * 1024
 
@@ -17,7 +15,7 @@ def folder(tmp_path_factory):
 
 @pytest.mark.parametrize("n_tt", [20, 56, 60])
 def test_an_accepted_plan_can_launch_its_gather(folder, n_tt):
-    bands, smem, terms = host_plan_sizes(many_edge_terms(n_tt), 64, 2, folder)
+    bands, smem, terms = gather_sizes(many_edge_terms(n_tt), 64, 2, folder)
     assert bands == 512 or smem <= 108 * 1024
     # 501 terms a sensor (more where tip/tilt removal adds its own), 8 bytes each beside the row's nodes
     assert (terms * 8 + 512 * 8 > LIMIT) == (n_tt >= 56)
