@@ -87,11 +87,18 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 // formed once for the corner rows above and below it: RS + 1 node rows are read
 // per layer instead of 2 RS, all requested before any is used.
 //
-// RS = kFwdStrip (4, FP64 2: kFwdThreads threads) for big launches, RS = 1 (more
-// warps, no reuse, less work in a chain) for small ones.  The steps that feed
-// the tile's partial sums (the slopes and the tip/tilt-only chunks) keep a
+// RS = kFwdStrip (4, FP64 2: kFwdThreads threads) for big launches, RS = 1 (a warp
+// per row, no reuse, less work in a chain) for small ones.  The steps that feed
+// the tile's partial sums (the slopes' sums and the tip/tilt-only chunks) keep a
 // fixed kFwdThreads-thread mapping, so the partials, and every result, are
-// bitwise the same at either block size.
+// bitwise the same at either block size.  In a small launch the slopes
+// themselves are formed by every warp, a row each, and taken to the four summing
+// warps through shared memory; there the loop over the layers and the pairs of a
+// tip/tilt-only chunk hold no branch, so all their loads are in flight at once.
+// Normal operator of one system (GB300, us): four warps forming the slopes, a
+// break after the last layer and a branch per pair 20.1, this form 19.3 (9 layers
+// of 64 x 64, 9 sensors); 19.7 and 18.7 (7 layers, 7 sensors); 17.7 and 16.8 (8
+// layers of 32 x 32, 6 sensors).
 //
 // Bound by instruction issue and L1 in big launches, by latency in small ones.
 // Against one corner per thread on 18 x 18 corners, four loads per corner and
@@ -121,6 +128,11 @@ __host__ __device__ constexpr size_t fwd_table_bytes(int L) {
   return L * (kFwdPsi<T> * sizeof(FwdRow<T>) + kFwdLanes * sizeof(T) + (kFwdLanes + 2) * sizeof(int)) + 16;
 }
 
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // (1 - f) a + f b, rounded the same way wherever it is used.
 __device__ __forceinline__ float lerp(float f, float a, float b) {
   return __fmaf_rn(__fsub_rn(1.f, f), a, __fmul_rn(f, b));
@@ -137,8 +149,32 @@ __device__ __forceinline__ void trace_strip(const T *__restrict__ phi, int L, in
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int j = 0; j < RS; ++j) val[j] = T(0);
+  if constexpr (RS == 1) {
+    // four layers' loads in flight, the sums predicated rather than left by a break
+    for (int l0 = 0; l0 < L; l0 += 4) {
+      T v00[4], v01[4], v10[4], v11[4], fx[4], fy[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int l = l0 + q < L ? l0 + q : L - 1;
+        const int N = s_N[l], x0 = s_x0[l * kFwdLanes + lane];
+        const FwdRow<T> row = s_row[l * kFwdPsi<T> + w];
+        const int x1 = (x0 + 1) & (N - 1), y1 = (row.y0 + 1) & (N - 1);
+        const T *p = phi + s_off[l];
+        fx[q] = s_fx[l * kFwdLanes + lane];
+        fy[q] = row.f;
+        v00[q] = p[row.y0 * N + x0];
+        v01[q] = p[row.y0 * N + x1];
+        v10[q] = p[y1 * N + x0];
+        v11[q] = p[y1 * N + x1];
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (l0 + q < L) val[0] += lerp(fy[q], lerp(fx[q], v00[q], v01[q]), lerp(fx[q], v10[q], v11[q]));
+    }
+    return;
+  }
   // layers whose loads are in flight together
-  constexpr int kBatch = RS == 1 ? 4 : 2;
+  constexpr int kBatch = 2;
   for (int l0 = 0; l0 < L; l0 += kBatch) {
     T v0[kBatch][RS + 1], v1[kBatch][RS + 1], fx[kBatch], fy[kBatch][RS];
     int r0[kBatch][RS];
@@ -169,7 +205,7 @@ __device__ __forceinline__ void trace_strip(const T *__restrict__ phi, int L, in
         last = r1;
       }
     }
-    const bool skips = RS > 1 && __any_sync(0xffffffffu, odd);   // (the same in every lane)
+    const bool skips = __any_sync(0xffffffffu, odd);   // (the same in every lane)
 #pragma unroll
     for (int q = 0; q < kBatch; ++q) {
       if (l0 + q >= L) break;
@@ -201,6 +237,9 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
   __shared__ T s_psi[kFwdPsi<T>][kFwdLanes + 1];
   __shared__ T s_ex[kFwdRows<T> + 1][kFwdLanes];
   __shared__ T s_ey[kFwdRows<T> + 1][kFwdLanes];
+  // the slopes of a small launch, formed by every warp, for the four summing warps
+  constexpr bool kAllWarps = RS == 1;
+  __shared__ T s_z[2][kAllWarps ? kFwdRows<T> + 1 : 1][kFwdLanes];
   pdl_trigger();
   const FwdItem it = items[blockIdx.x];
   if (io.active && !io.active[it.inst]) return;
@@ -266,42 +305,59 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
       }
       return;
     }
+    // (no branch between a thread's pairs, the indices clamped: every pair's edge corner is requested
+    // before any is used, then every pair's tables, then every pair's grid values)
     constexpr int U = kFwdChunk / kFwdThreads;
+    const int pairs = W.n_edge * L;
     int at[U][4];
     T fx[U], fy[U], tx[U], ty[U];
-    bool on[U];
+    if (tid < kFwdThreads) {
+      int c[U], lay[U], x0[U], y0[U], N[U], off[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int pair = it.tile * kFwdChunk + u * kFwdThreads + tid;
-      on[u] = tid < kFwdThreads && pair < W.n_edge * L;
-      if (!on[u]) continue;
-      const int e = pair / L, l = pair - e * L;
-      const int c = I.edge_idx[W.edge_off + e];
-      const int a = c % nc, b = c / nc;
-      const T *et = static_cast<const T *>(I.edge_t) + 2 * (W.edge_off + e);
-      const int po = 2 * l * nc, N = I.layers[l].N, off = I.layers[l].off;
-      const int x0 = pi[po + a], y0 = pi[po + nc + b];
-      const int x1 = (x0 + 1) & (N - 1), y1 = (y0 + 1) & (N - 1);
-      at[u][0] = off + y0 * N + x0;
-      at[u][1] = off + y0 * N + x1;
-      at[u][2] = off + y1 * N + x0;
-      at[u][3] = off + y1 * N + x1;
-      fx[u] = pf[po + a];
-      fy[u] = pf[po + nc + b];
-      tx[u] = et[0];
-      ty[u] = et[1];
+      for (int u = 0; u < U; ++u) {
+        const int pair = min(it.tile * kFwdChunk + u * kFwdThreads + tid, pairs - 1), e = pair / L;
+        const T *et = static_cast<const T *>(I.edge_t) + 2 * (W.edge_off + e);
+        lay[u] = pair - e * L;
+        c[u] = I.edge_idx[W.edge_off + e];
+        tx[u] = et[0];
+        ty[u] = et[1];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int b = c[u] / nc, a = c[u] - b * nc, po = 2 * lay[u] * nc;
+        x0[u] = pi[po + a];
+        y0[u] = pi[po + nc + b];
+        fx[u] = pf[po + a];
+        fy[u] = pf[po + nc + b];
+        N[u] = I.layers[lay[u]].N;
+        off[u] = I.layers[lay[u]].off;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int x1 = (x0[u] + 1) & (N[u] - 1), y1 = (y0[u] + 1) & (N[u] - 1);
+        at[u][0] = off[u] + y0[u] * N[u] + x0[u];
+        at[u][1] = off[u] + y0[u] * N[u] + x1;
+        at[u][2] = off[u] + y1 * N[u] + x0[u];
+        at[u][3] = off[u] + y1 * N[u] + x1;
+      }
     }
     pdl_wait();
     Acc<T> ax, ay;
+    if (tid < kFwdThreads) {
+      T g[U][4];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (on[u]) {
-        const T v00 = phi[at[u][0]], v01 = phi[at[u][1]];
-        const T v10 = phi[at[u][2]], v11 = phi[at[u][3]];
-        const T ps = lerp(fy[u], lerp(fx[u], v00, v01), lerp(fx[u], v10, v11));
-        ax.add_prod(tx[u], ps);
-        ay.add_prod(ty[u], ps);
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) g[u][q] = phi[at[u][q]];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const T ps = lerp(fy[u], lerp(fx[u], g[u][0], g[u][1]), lerp(fx[u], g[u][2], g[u][3]));
+        if (it.tile * kFwdChunk + u * kFwdThreads + tid < pairs) {
+          ax.add_prod(tx[u], ps);
+          ay.add_prod(ty[u], ps);
+        }
       }
+    }
     store_tile_partial(part + 2 * it.tile, ax, ay);
     return;
   }
@@ -336,14 +392,13 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
   const int *sidx = I.sub_idx + W.sub_off;
   const int lane = tid & 31, warp = tid >> 5;
   // the slope indices of step 2 (constant: before the dependency wait)
-  constexpr int kSubRounds = (kFwdRows<T> + kFwdThreads / 32) / (kFwdThreads / 32);
+  constexpr int kSumWarps = kFwdThreads / 32, kSumRounds = (kFwdRows<T> + kSumWarps) / kSumWarps;
+  constexpr int kSubWarps = kFwdPsi<T> / RS, kSubRounds = (kFwdRows<T> + kSubWarps) / kSubWarps;
   int sj[kSubRounds];
 #pragma unroll
   for (int q = 0; q < kSubRounds; ++q) {
-    const int w = warp + q * (kFwdThreads / 32), a = a0 - 1 + lane, b = b0 - 1 + w;
-    sj[q] = tid < kFwdThreads && lane <= kFwdCols && w <= kFwdRows<T> && a >= 0 && b >= 0 && a < n && b < n
-                ? sidx[b * n + a]
-                : -1;
+    const int w = warp + q * kSubWarps, a = a0 - 1 + lane, b = b0 - 1 + w;
+    sj[q] = lane <= kFwdCols && w <= kFwdRows<T> && a >= 0 && b >= 0 && a < n && b < n ? sidx[b * n + a] : -1;
   }
   // 1. psi on the tile's corners plus a one-corner halo
   {
@@ -367,23 +422,24 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
     for (int j = 0; j < RS; ++j) s_psi[w + j][lane] = on[j] ? val[j] : T(0);
   }
   __syncthreads();
-  // 2. weighted slopes of the subapertures the tile's corners touch: four warps, one lane per column
+  // 2. weighted slopes of the subapertures the tile's corners touch, one lane per column
   Acc<T> sx_acc, sy_acc, qx_acc, qy_acc;
   const T isg = sizeof(T) == 4 ? T(W.inv_sigma2_f) : T(W.inv_sigma2);   // no FP64 conversion in FP32
   // spot elongation: the block sigma^2 (I + tau g g^T) is inverted in closed
   // form, sigma^-2 (I - c g g^T) with c = tau / (1 + tau |g|^2)
   const bool elong = EL && W.elong != 0;
   const T el_tau = EL ? T(W.el_tau) : T(0), el_eps = EL ? T(W.el_eps) : T(0), el_d = EL ? T(W.d_sub) : T(0);
-  const T el_cx = EL ? T(0.5 - 0.5 * n) * el_d - T(W.el_lx) : T(0);
-  const T el_cy = EL ? T(0.5 - 0.5 * n) * el_d - T(W.el_ly) : T(0);
+  const T el_cx = EL ? fma_rn(T(0.5 - 0.5 * n), el_d, -T(W.el_lx)) : T(0);
+  const T el_cy = EL ? fma_rn(T(0.5 - 0.5 * n), el_d, -T(W.el_ly)) : T(0);
   const bool four = EL && tile_partials(W) == 4;
-  if (tid < kFwdThreads && lane <= kFwdCols) {
+  const bool sums = W.kind == kRemoveTT;
+  if (lane <= kFwdCols) {
     const int u = lane, a = a0 - 1 + u;
 #pragma unroll
     for (int q = 0; q < kSubRounds; ++q) {
-      const int w = warp + q * (kFwdThreads / 32), b = b0 - 1 + w, j = sj[q];
+      const int w = warp + q * kSubWarps, b = b0 - 1 + w, j = sj[q];
       if (w > kFwdRows<T>) break;
-      T ex = T(0), ey = T(0);
+      T ex = T(0), ey = T(0), zx = T(0), zy = T(0);
       if (j >= 0) {
         const T p00 = s_psi[w][u], p10 = s_psi[w][u + 1];
         const T p01 = s_psi[w + 1][u], p11 = s_psi[w + 1][u + 1];
@@ -405,16 +461,20 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
           sy = dat[W.slope_off + W.S + j];
         }
         if (elong) {
-          const T gx = el_eps * (T(a) * el_d + el_cx), gy = el_eps * (T(b) * el_d + el_cy);
-          const T c = el_tau / (T(1) + el_tau * (gx * gx + gy * gy));
-          const T dot = c * (gx * sx + gy * sy);
-          ex = isg * (sx - gx * dot);
-          ey = isg * (sy - gy * dot);
+          // (every rounding stated: the compiler contracts products differently from one instance to another)
+          const T gx = mul_rn(el_eps, fma_rn(T(a), el_d, el_cx)), gy = mul_rn(el_eps, fma_rn(T(b), el_d, el_cy));
+          const T c = el_tau / fma_rn(el_tau, fma_rn(gx, gx, mul_rn(gy, gy)), T(1));
+          const T dot = mul_rn(c, fma_rn(gx, sx, mul_rn(gy, sy)));
+          ex = mul_rn(isg, fma_rn(-gx, dot, sx));
+          ey = mul_rn(isg, fma_rn(-gy, dot, sy));
         } else {
           ex = isg * sx;
           ey = isg * sy;
         }
-        if (u >= 1 && w >= 1) {   // subapertures owned by this tile
+        if (kAllWarps) {
+          zx = sx;
+          zy = sy;
+        } else if (u >= 1 && w >= 1) {   // subapertures owned by this tile
           sx_acc.add(sx);
           sy_acc.add(sy);
           if (four) {
@@ -425,10 +485,28 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
       }
       s_ex[w][u] = ex;
       s_ey[w][u] = ey;
+      if (kAllWarps && sums) {
+        s_z[0][w][u] = zx;
+        s_z[1][w][u] = zy;
+      }
     }
   }
   if (MODE == 3) return;
   __syncthreads();
+  if (kAllWarps && sums && warp < kSumWarps && lane >= 1 && lane <= kFwdCols) {
+    // the owned subapertures' z (zero where there is none) on the four warps, rows in the order above
+#pragma unroll
+    for (int q = 0; q < kSumRounds; ++q) {
+      const int w = warp + q * kSumWarps;
+      if (w < 1 || w > kFwdRows<T>) continue;
+      sx_acc.add(s_z[0][w][lane]);
+      sy_acc.add(s_z[1][w][lane]);
+      if (four) {
+        qx_acc.add(s_ex[w][lane]);
+        qy_acc.add(s_ey[w][lane]);
+      }
+    }
+  }
   // 3. Gamma^T: each corner gathers its four neighbouring subapertures
   if (lane < kFwdCols) {
     const int u = lane, a = a0 + u;
@@ -441,7 +519,7 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
       }
     }
   }
-  if (W.kind != kRemoveTT) return;
+  if (!sums) return;
   // 4. tip/tilt removal: this tile's sums of z (the consumer forms the means)
   if (four) {
     store_tile_partial(part + 4 * it.tile, sx_acc, sy_acc);

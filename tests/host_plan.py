@@ -28,3 +28,9 @@ def gather_sizes(geom, cluster_size, transforms, folder):
 def coarse_sides(geom, cluster_size, transforms, folder):
     """Per layer, the side of the block that one CTA of its cluster finishes."""
     return _call("host_plan_coarse", geom, cluster_size, transforms, folder, len(geom["layers"]))
+
+
+def forward_ctas(geom, cluster_size, transforms, folder):
+    """(CTAs of one forward launch, CTAs up to which a launch takes the small form)."""
+    n = _call("host_plan_forward", geom, cluster_size, transforms, folder, 1)[0]
+    return n, ctypes.CDLL(os.path.join(str(folder), "libhostplan.so")).host_plan_forward_small()

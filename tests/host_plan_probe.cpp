@@ -28,3 +28,15 @@ extern "C" int host_plan_coarse(const tomo_geometry *g, int cluster_size, int tr
   for (size_t l = 0; l < P.layers.size(); ++l) out[l] = P.layers[l].coarse;
   return TOMO_OK;
 }
+
+// out[0]: CTAs of one forward launch (tiles of the sensors, chunks of the tip/tilt-only ones).
+extern "C" int host_plan_forward(const tomo_geometry *g, int cluster_size, int transforms, long long *out) {
+  tomo::HostPlan P;
+  std::string err;
+  const int st = tomo::build_host_plan(g, &P, &err, cluster_size, transforms);
+  if (st == TOMO_OK) out[0] = static_cast<long long>(P.fwd_items.size());
+  return st;
+}
+
+// CTAs up to which a forward launch takes the small form.
+extern "C" int host_plan_forward_small() { return tomo::kFwdSmallLaunch; }
