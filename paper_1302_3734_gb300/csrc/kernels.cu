@@ -104,7 +104,21 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 // Against one corner per thread on 18 x 18 corners, four loads per corner and
 // layer (GB300, cold launch): 16 E-ELT systems 49.2 -> 29 us, 64 uneven systems
 // 50.9 -> 29 us, the 100 m system 54.0 -> 43 us.
-constexpr size_t kFwdSmallSmem = 64 * 1024;
+// The kernels of a frame overlap by programmatic launch: an analysis CTA (up to 108 KB) can start
+// beside the forward CTAs only if the SM's split between L1 and shared memory holds both.  A forward
+// CTA alone (about 14 KB) asks for a small split; small launches ask for 72% (164 KB, which leaves
+// 64 KB of L1).  59 systems of 9 to 120 subapertures, FP32, geometric means of the time (GB300, one
+// sweep) against 64 KB of unused shared memory per CTA, normal operator and solve of 10 iterations:
+// 50% 1.003 and 0.996, 72% 0.992 and 0.993, 86% 0.999 and 0.997; in another sweep nothing 0.999 and
+// 1.001, 72% 0.999 and 0.993.  E-ELT frame, us: nothing 414, 64 KB 408, 72% 409.
+constexpr int kFwdCarveout = 72;
+// FP64: an SM's FP64 pipe is slow enough that CTAs sharing an SM while others are idle cost more
+// than anything, so a launch of up to one and a half CTAs per SM of 152 asks for 100 KB each: one
+// forward CTA per SM.  Normal operator (us, without and with): 4 sensors of 88 x 88 (180 CTAs) 77
+// and 59, 6 of 60 x 60 (200) 108 and 104, 6 of 31 x 31 57 and 44; 6 of 84 x 84 (300 CTAs) would
+// go from 122 to 126.
+constexpr size_t kFwdAloneSmem = 100 * 1024;
+constexpr int kFwdAloneLaunch = 228;
 constexpr int kFwdLanes = kFwdCols + 2;
 template <typename T>
 constexpr int kFwdRows = fwd_rows(sizeof(T) == 8);
@@ -1663,22 +1677,25 @@ cudaError_t allow_type() {
   if (e == cudaSuccess) e = allow_lf<T, 4>();
   if (e == cudaSuccess) e = allow_lf<T, 6>();
   if (e == cudaSuccess) e = allow_lf<T, 8>();
-  const void *fwd[14] = {reinterpret_cast<const void *>(k_forward<T, 0, false, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, false, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, false, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 0, true, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, true, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, true, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 0, false, kFwdStrip<T>>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, false, kFwdStrip<T>>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, false, kFwdStrip<T>>),
-                         reinterpret_cast<const void *>(k_forward<T, 0, true, kFwdStrip<T>>),
-                         reinterpret_cast<const void *>(k_forward<T, 1, true, kFwdStrip<T>>),
-                         reinterpret_cast<const void *>(k_forward<T, 2, true, kFwdStrip<T>>),
-                         reinterpret_cast<const void *>(k_forward<T, 3, false, 1>),
-                         reinterpret_cast<const void *>(k_forward<T, 3, false, kFwdStrip<T>>)};
+  const void *fwd[14] = {   // the small launches' forms first
+      reinterpret_cast<const void *>(k_forward<T, 0, false, 1>),
+      reinterpret_cast<const void *>(k_forward<T, 1, false, 1>),
+      reinterpret_cast<const void *>(k_forward<T, 2, false, 1>),
+      reinterpret_cast<const void *>(k_forward<T, 0, true, 1>),
+      reinterpret_cast<const void *>(k_forward<T, 1, true, 1>),
+      reinterpret_cast<const void *>(k_forward<T, 2, true, 1>),
+      reinterpret_cast<const void *>(k_forward<T, 3, false, 1>),
+      reinterpret_cast<const void *>(k_forward<T, 0, false, kFwdStrip<T>>),
+      reinterpret_cast<const void *>(k_forward<T, 1, false, kFwdStrip<T>>),
+      reinterpret_cast<const void *>(k_forward<T, 2, false, kFwdStrip<T>>),
+      reinterpret_cast<const void *>(k_forward<T, 0, true, kFwdStrip<T>>),
+      reinterpret_cast<const void *>(k_forward<T, 1, true, kFwdStrip<T>>),
+      reinterpret_cast<const void *>(k_forward<T, 2, true, kFwdStrip<T>>),
+      reinterpret_cast<const void *>(k_forward<T, 3, false, kFwdStrip<T>>)};
   for (int i = 0; i < 14 && e == cudaSuccess; ++i)
     e = cudaFuncSetAttribute(fwd[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxForwardSmem);
+  for (int i = 0; i < 7 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(fwd[i], cudaFuncAttributePreferredSharedMemoryCarveout, kFwdCarveout);
   return e;
 }
 
@@ -1788,12 +1805,8 @@ cudaError_t fwd_t(int mode, dim3 g, size_t sm, cudaStream_t s, const InstDev *in
 cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, const InstDev *insts,
                            const FwdItem *items, int n_items, const IoArgs &io, cudaStream_t s) {
   const dim3 g(n_items);
-  // A small launch asks for more shared memory than its tables need: with 64 KB per CTA no two of
-  // the analysis kernel's CTAs (about 100 KB) start on one SM beside a forward CTA while other SMs
-  // have none (programmatic launch places them early).  E-ELT frame, us by KB per CTA: 420 (none),
-  // 414 (64), 414 (80), 419 (100), 434 (120).
   const size_t need = forward_smem(max_layers, precision);
-  const size_t sm = n_items <= kFwdSmallLaunch && need < kFwdSmallSmem ? kFwdSmallSmem : need;
+  const size_t sm = precision && n_items <= kFwdAloneLaunch && need < kFwdAloneSmem ? kFwdAloneSmem : need;
   if (precision == 0)
     return elong ? fwd_t<float, true>(mode, g, sm, s, insts, items, io)
                  : fwd_t<float, false>(mode, g, sm, s, insts, items, io);
