@@ -106,6 +106,8 @@ cudaError_t anal_ls(const LaunchSet &L, int src, int epi, int flags, const IoArg
   return L.stream ? launch_analysis_streamed(L.precision, src, epi, L.lf, flags, L.d_inst, L.ss, io, s)
                   : launch_analysis(L.precision, src, epi, L.lf, flags, L.d_inst, L.cl, L.n_cl, L.C, L.smem_a, io, s);
 }
+// Shared memory of the analysis CTAs that start beside the forward kernel's (streamed plans: none do).
+size_t beside(const LaunchSet &L) { return L.stream ? 0 : L.smem_a; }
 int anal_launches(const LaunchSet &L) { return L.stream ? streamed_launches(L.ss) : 1; }
 
 // The gather of the plan's corner fields and W of the result with epilogue epi
@@ -143,7 +145,7 @@ tomo_status enqueue_solve(tomo_plan *tp, const LaunchSet &L, const void *const *
     io.active = active;
     for (int i = 0; i < L.count; ++i) io.in1[i] = slopes[i];
     TOMO_TRY(timed(tp, kKindFwd, s, [&] {
-      return launch_forward(L.precision, warm ? 1 : 2, L.max_layers, L.elong, L.d_inst, L.fwd, L.n_fwd, io, s);
+      return launch_forward(L.precision, warm ? 1 : 2, L.max_layers, L.elong, beside(L), L.d_inst, L.fwd, L.n_fwd, io, s);
     }, "forward (residual)"));
     ++nk;
   }
@@ -176,7 +178,7 @@ tomo_status enqueue_solve(tomo_plan *tp, const LaunchSet &L, const void *const *
       return synthesis_of(L, 1, (it == 0 ? kFlagFirst : 0) | (it << kIterShift), none, s);
     }, "synthesis", synthesis_launches(L)));
     TOMO_TRY(timed(tp, kKindFwd, s, [&] {
-      return launch_forward(L.precision, 0, L.max_layers, L.elong, L.d_inst, L.fwd, L.n_fwd, none, s);
+      return launch_forward(L.precision, 0, L.max_layers, L.elong, beside(L), L.d_inst, L.fwd, L.n_fwd, none, s);
     }, "forward"));
     if (L.split) {
       TOMO_TRY(timed(tp, kKindGather, s, [&] {
@@ -1005,7 +1007,7 @@ tomo_status tomo_layers_to_slopes(tomo_plan *p, const void *d_layers, void *d_sl
   io.out0[0] = d_slopes;
   return timed(p, kKindOther, s, [&] {
     const LaunchSet &L = p->ls;
-    return launch_forward(L.precision, 3, L.max_layers, 0, L.d_inst, L.fwd, L.n_fwd, io, s);
+    return launch_forward(L.precision, 3, L.max_layers, 0, beside(L), L.d_inst, L.fwd, L.n_fwd, io, s);
   }, "slopes");
 }
 
@@ -1020,7 +1022,7 @@ tomo_status tomo_apply_normal(tomo_plan *p, const void *d_in, void *d_out, void 
   a.in0[0] = d_in;
   TOMO_TRY(timed(p, kKindSynth, s, [&] { return synthesis_of(L, 0, 0, a, s); }, "synthesis", synthesis_launches(L)));
   IoArgs b{};
-  TOMO_TRY(timed(p, kKindFwd, s, [&] { return launch_forward(L.precision, 0, L.max_layers, L.elong, L.d_inst, L.fwd, L.n_fwd, b, s); },
+  TOMO_TRY(timed(p, kKindFwd, s, [&] { return launch_forward(L.precision, 0, L.max_layers, L.elong, beside(L), L.d_inst, L.fwd, L.n_fwd, b, s); },
                  "forward"));
   IoArgs c{};
   c.in1[0] = d_in;
@@ -1036,7 +1038,7 @@ tomo_status tomo_rhs(tomo_plan *p, const void *d_slopes, void *d_out, void *cuda
   const LaunchSet &L = p->ls;
   IoArgs a{};
   a.in1[0] = d_slopes;
-  TOMO_TRY(timed(p, kKindFwd, s, [&] { return launch_forward(L.precision, 2, L.max_layers, L.elong, L.d_inst, L.fwd, L.n_fwd, a, s); },
+  TOMO_TRY(timed(p, kKindFwd, s, [&] { return launch_forward(L.precision, 2, L.max_layers, L.elong, beside(L), L.d_inst, L.fwd, L.n_fwd, a, s); },
                  "forward (data)"));
   IoArgs c{};
   c.out0[0] = d_out;

@@ -29,6 +29,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "common.h"
 #include "device_util.cuh"
 #include "launch.h"
@@ -91,12 +93,15 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 // per row, no reuse, less work in a chain) for small ones.  The steps that feed
 // the tile's partial sums (the slopes' sums and the tip/tilt-only chunks) keep a
 // fixed kFwdThreads-thread mapping, so the partials, and every result, are
-// bitwise the same at either block size.  In a small launch the slopes
-// themselves are formed by every warp, a row each, and taken to the four summing
-// warps through shared memory; there the loop over the layers and the pairs of a
-// tip/tilt-only chunk hold no branch, so all their loads are in flight at once.
+// bitwise the same at either block size.  In a small launch without elongated
+// spots the slopes themselves are formed by every warp, a row each, and taken to
+// the four summing warps through shared memory (with elongated spots, whose
+// sums are four, that costs more than it saves: 114 x 114, one layer, 22.8 ->
+// 23.6 us an operator); the loop over the layers and the pairs of a tip/tilt-only
+// chunk hold no branch, so all their loads are in flight at once, and a last
+// layer alone is not padded to a batch of four (E-ELT solve 409 -> 403 us).
 // Normal operator of one system (GB300, us): four warps forming the slopes, a
-// break after the last layer and a branch per pair 20.1, this form 19.3 (9 layers
+// break after the last layer and a branch per pair 20.0, this form 19.1 (9 layers
 // of 64 x 64, 9 sensors); 19.7 and 18.7 (7 layers, 7 sensors); 17.7 and 16.8 (8
 // layers of 32 x 32, 6 sensors).
 //
@@ -104,14 +109,19 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 // Against one corner per thread on 18 x 18 corners, four loads per corner and
 // layer (GB300, cold launch): 16 E-ELT systems 49.2 -> 29 us, 64 uneven systems
 // 50.9 -> 29 us, the 100 m system 54.0 -> 43 us.
-// The kernels of a frame overlap by programmatic launch: an analysis CTA (up to 108 KB) can start
-// beside the forward CTAs only if the SM's split between L1 and shared memory holds both.  A forward
-// CTA alone (about 14 KB) asks for a small split; small launches ask for 72% (164 KB, which leaves
-// 64 KB of L1).  59 systems of 9 to 120 subapertures, FP32, geometric means of the time (GB300, one
-// sweep) against 64 KB of unused shared memory per CTA, normal operator and solve of 10 iterations:
-// 50% 1.003 and 0.996, 72% 0.992 and 0.993, 86% 0.999 and 0.997; in another sweep nothing 0.999 and
-// 1.001, 72% 0.999 and 0.993.  E-ELT frame, us: nothing 414, 64 KB 408, 72% 409.
+// What a small launch asks of an SM.  The kernels of a frame overlap by programmatic launch: an
+// analysis CTA (up to 108 KB) can start beside the forward CTAs only if the SM's split between L1
+// and shared memory holds both.  A forward CTA alone (about 14 KB) asks for a small split; small
+// launches ask for 72% (164 KB, which leaves 64 KB of L1).  59 systems of 9 to 120 subapertures,
+// FP32, geometric means of the time (GB300) against 64 KB of unused shared memory per CTA and the
+// driver's split, normal operator and solve of 10 iterations: 50% 1.003 and 0.996, 72% 0.992 and
+// 0.993, 86% 0.999 and 0.997; neither 0.999 and 1.001.
+// Where an analysis CTA takes 64 KB itself, so that where it starts matters more, each forward CTA
+// takes 64 KB as well (at 72%, us without and with: 67 x 67, 3 layers 36.1 and 32.6 an operator;
+// 104 x 104, 5 layers 26.6 and 26.2, and 399 and 390 a solve; E-ELT 31.9 and 31.7; smaller analysis
+// CTAs lose: 82 x 82, 1 layer 300 and 314 a solve, 64 x 64, 5 layers 274 and 292).
 constexpr int kFwdCarveout = 72;
+constexpr size_t kFwdBesideSmem = 64 * 1024;
 // FP64: an SM's FP64 pipe is slow enough that CTAs sharing an SM while others are idle cost more
 // than anything, so a launch of up to one and a half CTAs per SM of 152 asks for 100 KB each: one
 // forward CTA per SM.  Normal operator (us, without and with): 4 sensors of 88 x 88 (180 CTAs) 77
@@ -164,11 +174,12 @@ __device__ __forceinline__ void trace_strip(const T *__restrict__ phi, int L, in
 #pragma unroll
   for (int j = 0; j < RS; ++j) val[j] = T(0);
   if constexpr (RS == 1) {
-    // four layers' loads in flight, the sums predicated rather than left by a break
-    for (int l0 = 0; l0 < L; l0 += 4) {
-      T v00[4], v01[4], v10[4], v11[4], fx[4], fy[4];
+    // NB layers from l0, their loads in flight together, the sums predicated rather than left by a break
+    auto batch = [&](int l0, auto nb) {
+      constexpr int NB = decltype(nb)::value;
+      T v00[NB], v01[NB], v10[NB], v11[NB], fx[NB], fy[NB];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < NB; ++q) {
         const int l = l0 + q < L ? l0 + q : L - 1;
         const int N = s_N[l], x0 = s_x0[l * kFwdLanes + lane];
         const FwdRow<T> row = s_row[l * kFwdPsi<T> + w];
@@ -182,9 +193,12 @@ __device__ __forceinline__ void trace_strip(const T *__restrict__ phi, int L, in
         v11[q] = p[y1 * N + x1];
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int q = 0; q < NB; ++q)
         if (l0 + q < L) val[0] += lerp(fy[q], lerp(fx[q], v00[q], v01[q]), lerp(fx[q], v10[q], v11[q]));
-    }
+    };
+    int l0 = 0;
+    for (; l0 + 1 < L; l0 += 4) batch(l0, std::integral_constant<int, 4>());
+    if (l0 < L) batch(l0, std::integral_constant<int, 1>());   // (a last layer alone: no loads for padding)
     return;
   }
   // layers whose loads are in flight together
@@ -252,7 +266,7 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
   __shared__ T s_ex[kFwdRows<T> + 1][kFwdLanes];
   __shared__ T s_ey[kFwdRows<T> + 1][kFwdLanes];
   // the slopes of a small launch, formed by every warp, for the four summing warps
-  constexpr bool kAllWarps = RS == 1;
+  constexpr bool kAllWarps = RS == 1 && !EL;
   __shared__ T s_z[2][kAllWarps ? kFwdRows<T> + 1 : 1][kFwdLanes];
   pdl_trigger();
   const FwdItem it = items[blockIdx.x];
@@ -319,58 +333,95 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
       }
       return;
     }
-    // (no branch between a thread's pairs, the indices clamped: every pair's edge corner is requested
-    // before any is used, then every pair's tables, then every pair's grid values)
     constexpr int U = kFwdChunk / kFwdThreads;
     const int pairs = W.n_edge * L;
     int at[U][4];
     T fx[U], fy[U], tx[U], ty[U];
-    if (tid < kFwdThreads) {
-      int c[U], lay[U], x0[U], y0[U], N[U], off[U];
+    Acc<T> ax, ay;
+    if constexpr (RS == 1) {
+      // no branch between a thread's pairs, the indices clamped: every pair's edge corner is requested
+      // before any is used, then every pair's tables, then every pair's grid values (in big launches
+      // the SM's other CTAs hide these latencies and the clamped form costs 0.7%: 16 E-ELT systems
+      // 1139 -> 1149 us)
+      if (tid < kFwdThreads) {
+        int c[U], lay[U], x0[U], y0[U], N[U], off[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int pair = min(it.tile * kFwdChunk + u * kFwdThreads + tid, pairs - 1), e = pair / L;
+          const T *et = static_cast<const T *>(I.edge_t) + 2 * (W.edge_off + e);
+          lay[u] = pair - e * L;
+          c[u] = I.edge_idx[W.edge_off + e];
+          tx[u] = et[0];
+          ty[u] = et[1];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int b = c[u] / nc, a = c[u] - b * nc, po = 2 * lay[u] * nc;
+          x0[u] = pi[po + a];
+          y0[u] = pi[po + nc + b];
+          fx[u] = pf[po + a];
+          fy[u] = pf[po + nc + b];
+          N[u] = I.layers[lay[u]].N;
+          off[u] = I.layers[lay[u]].off;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int x1 = (x0[u] + 1) & (N[u] - 1), y1 = (y0[u] + 1) & (N[u] - 1);
+          at[u][0] = off[u] + y0[u] * N[u] + x0[u];
+          at[u][1] = off[u] + y0[u] * N[u] + x1;
+          at[u][2] = off[u] + y1 * N[u] + x0[u];
+          at[u][3] = off[u] + y1 * N[u] + x1;
+        }
+      }
+      pdl_wait();
+      if (tid < kFwdThreads) {
+        T g[U][4];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) g[u][q] = phi[at[u][q]];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const T ps = lerp(fy[u], lerp(fx[u], g[u][0], g[u][1]), lerp(fx[u], g[u][2], g[u][3]));
+          if (it.tile * kFwdChunk + u * kFwdThreads + tid < pairs) {
+            ax.add_prod(tx[u], ps);
+            ay.add_prod(ty[u], ps);
+          }
+        }
+      }
+    } else {
+      bool on[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int pair = min(it.tile * kFwdChunk + u * kFwdThreads + tid, pairs - 1), e = pair / L;
+        const int pair = it.tile * kFwdChunk + u * kFwdThreads + tid;
+        on[u] = pair < pairs;
+        if (!on[u]) continue;
+        const int e = pair / L, l = pair - e * L;
+        const int c = I.edge_idx[W.edge_off + e];
+        const int a = c % nc, b = c / nc;
         const T *et = static_cast<const T *>(I.edge_t) + 2 * (W.edge_off + e);
-        lay[u] = pair - e * L;
-        c[u] = I.edge_idx[W.edge_off + e];
+        const int po = 2 * l * nc, N = I.layers[l].N, off = I.layers[l].off;
+        const int x0 = pi[po + a], y0 = pi[po + nc + b];
+        const int x1 = (x0 + 1) & (N - 1), y1 = (y0 + 1) & (N - 1);
+        at[u][0] = off + y0 * N + x0;
+        at[u][1] = off + y0 * N + x1;
+        at[u][2] = off + y1 * N + x0;
+        at[u][3] = off + y1 * N + x1;
+        fx[u] = pf[po + a];
+        fy[u] = pf[po + nc + b];
         tx[u] = et[0];
         ty[u] = et[1];
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int b = c[u] / nc, a = c[u] - b * nc, po = 2 * lay[u] * nc;
-        x0[u] = pi[po + a];
-        y0[u] = pi[po + nc + b];
-        fx[u] = pf[po + a];
-        fy[u] = pf[po + nc + b];
-        N[u] = I.layers[lay[u]].N;
-        off[u] = I.layers[lay[u]].off;
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int x1 = (x0[u] + 1) & (N[u] - 1), y1 = (y0[u] + 1) & (N[u] - 1);
-        at[u][0] = off[u] + y0[u] * N[u] + x0[u];
-        at[u][1] = off[u] + y0[u] * N[u] + x1;
-        at[u][2] = off[u] + y1 * N[u] + x0[u];
-        at[u][3] = off[u] + y1 * N[u] + x1;
-      }
-    }
-    pdl_wait();
-    Acc<T> ax, ay;
-    if (tid < kFwdThreads) {
-      T g[U][4];
+      pdl_wait();
 #pragma unroll
       for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) g[u][q] = phi[at[u][q]];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const T ps = lerp(fy[u], lerp(fx[u], g[u][0], g[u][1]), lerp(fx[u], g[u][2], g[u][3]));
-        if (it.tile * kFwdChunk + u * kFwdThreads + tid < pairs) {
+        if (on[u]) {
+          const T v00 = phi[at[u][0]], v01 = phi[at[u][1]];
+          const T v10 = phi[at[u][2]], v11 = phi[at[u][3]];
+          const T ps = lerp(fy[u], lerp(fx[u], v00, v01), lerp(fx[u], v10, v11));
           ax.add_prod(tx[u], ps);
           ay.add_prod(ty[u], ps);
         }
-      }
     }
     store_tile_partial(part + 2 * it.tile, ax, ay);
     return;
@@ -407,12 +458,15 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
   const int lane = tid & 31, warp = tid >> 5;
   // the slope indices of step 2 (constant: before the dependency wait)
   constexpr int kSumWarps = kFwdThreads / 32, kSumRounds = (kFwdRows<T> + kSumWarps) / kSumWarps;
-  constexpr int kSubWarps = kFwdPsi<T> / RS, kSubRounds = (kFwdRows<T> + kSubWarps) / kSubWarps;
+  constexpr int kSubWarps = kAllWarps ? kFwdPsi<T> / RS : kSumWarps;
+  constexpr int kSubRounds = (kFwdRows<T> + kSubWarps) / kSubWarps;
   int sj[kSubRounds];
 #pragma unroll
   for (int q = 0; q < kSubRounds; ++q) {
     const int w = warp + q * kSubWarps, a = a0 - 1 + lane, b = b0 - 1 + w;
-    sj[q] = lane <= kFwdCols && w <= kFwdRows<T> && a >= 0 && b >= 0 && a < n && b < n ? sidx[b * n + a] : -1;
+    sj[q] = warp < kSubWarps && lane <= kFwdCols && w <= kFwdRows<T> && a >= 0 && b >= 0 && a < n && b < n
+                ? sidx[b * n + a]
+                : -1;
   }
   // 1. psi on the tile's corners plus a one-corner halo
   {
@@ -447,7 +501,7 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
   const T el_cy = EL ? fma_rn(T(0.5 - 0.5 * n), el_d, -T(W.el_ly)) : T(0);
   const bool four = EL && tile_partials(W) == 4;
   const bool sums = W.kind == kRemoveTT;
-  if (lane <= kFwdCols) {
+  if (warp < kSubWarps && lane <= kFwdCols) {
     const int u = lane, a = a0 - 1 + u;
 #pragma unroll
     for (int q = 0; q < kSubRounds; ++q) {
@@ -508,17 +562,13 @@ __global__ void __launch_bounds__(32 * kFwdPsi<T> / RS, RS == 1 ? 2 : (sizeof(T)
   if (MODE == 3) return;
   __syncthreads();
   if (kAllWarps && sums && warp < kSumWarps && lane >= 1 && lane <= kFwdCols) {
-    // the owned subapertures' z (zero where there is none) on the four warps, rows in the order above
+    // the owned subapertures' z (zero where there is none) on the four warps, rows in the strips' order
 #pragma unroll
     for (int q = 0; q < kSumRounds; ++q) {
       const int w = warp + q * kSumWarps;
       if (w < 1 || w > kFwdRows<T>) continue;
       sx_acc.add(s_z[0][w][lane]);
       sy_acc.add(s_z[1][w][lane]);
-      if (four) {
-        qx_acc.add(s_ex[w][lane]);
-        qy_acc.add(s_ey[w][lane]);
-      }
     }
   }
   // 3. Gamma^T: each corner gathers its four neighbouring subapertures
@@ -1802,11 +1852,13 @@ cudaError_t fwd_t(int mode, dim3 g, size_t sm, cudaStream_t s, const InstDev *in
                                 : fwd_rs<T, EL, kFwdStrip<T>>(mode, g, sm, s, insts, items, io);
 }
 
-cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, const InstDev *insts,
-                           const FwdItem *items, int n_items, const IoArgs &io, cudaStream_t s) {
+cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, size_t smem_analysis,
+                           const InstDev *insts, const FwdItem *items, int n_items, const IoArgs &io, cudaStream_t s) {
   const dim3 g(n_items);
   const size_t need = forward_smem(max_layers, precision);
-  const size_t sm = precision && n_items <= kFwdAloneLaunch && need < kFwdAloneSmem ? kFwdAloneSmem : need;
+  size_t sm = need;
+  if (precision == 0 && n_items <= kFwdSmallLaunch && smem_analysis >= kFwdBesideSmem) sm = max(need, kFwdBesideSmem);
+  if (precision == 1 && n_items <= kFwdAloneLaunch) sm = max(need, kFwdAloneSmem);
   if (precision == 0)
     return elong ? fwd_t<float, true>(mode, g, sm, s, insts, items, io)
                  : fwd_t<float, false>(mode, g, sm, s, insts, items, io);

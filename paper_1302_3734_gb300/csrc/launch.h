@@ -53,9 +53,11 @@ cudaError_t configure_streamed_kernels();
 cudaError_t configure_gather_kernels();
 
 // Ray-trace, Fried slopes, noise weighting, Gamma^T.  mode 0 operator, 1 residual,
-// 2 data only, 3 the noise-free measurement of io.in0 into io.out0.  elong: some sensor of the launch has elongated spots.
-cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, const InstDev *insts,
-                           const FwdItem *items, int n_items, const IoArgs &io, cudaStream_t s);
+// 2 data only, 3 the noise-free measurement of io.in0 into io.out0.  elong: some sensor of the
+// launch has elongated spots; smem_analysis: shared memory of the analysis CTAs that
+// start beside this kernel's (0: none).
+cudaError_t launch_forward(int precision, int mode, int max_layers, int elong, size_t smem_analysis,
+                           const InstDev *insts, const FwdItem *items, int n_items, const IoArgs &io, cudaStream_t s);
 
 // x, r update of `count` instances and the FP64 r.z partials; flags carries the iteration
 // index.  update_launches: the kernels one call launches.
