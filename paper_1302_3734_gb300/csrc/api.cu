@@ -1007,7 +1007,7 @@ tomo_status tomo_layers_to_slopes(tomo_plan *p, const void *d_layers, void *d_sl
   io.out0[0] = d_slopes;
   return timed(p, kKindOther, s, [&] {
     const LaunchSet &L = p->ls;
-    return launch_forward(L.precision, 3, L.max_layers, 0, beside(L), L.d_inst, L.fwd, L.n_fwd, io, s);
+    return launch_forward(L.precision, 3, L.max_layers, 0, 0, L.d_inst, L.fwd, L.n_fwd, io, s);
   }, "slopes");
 }
 

@@ -17,7 +17,7 @@ constexpr int kFwdTile = 16;       // subapertures per side of a mirror-slope ti
 // (FP64 8 m frame of 30 iterations, GB300: 990 us against 1070 with 14 rows.)
 constexpr int kFwdCols = 30;
 constexpr int fwd_rows(int precision) { return precision ? 6 : 14; }
-constexpr int kFwdThreads = 128;   // threads of a forward CTA in big launches (four times that in small ones)
+constexpr int kFwdThreads = 128;   // threads of a forward CTA in big launches (small ones: 512, FP64 256)
 constexpr int kFwdChunk = 512;     // (edge corner, layer) pairs of a tip/tilt-only forward CTA
 constexpr int kMaxBatch = 96;      // instances per launch (kernel-argument arrays)
 constexpr int kThreads = 256;      // threads per CTA of the hot kernels (transforms: below)
@@ -205,8 +205,8 @@ TOMO_HD inline int tile_partials(const WfsDev &d) { return (d.elong && d.kind ==
 // Side of the low-low block from which CTA 0 of a cluster finishes a layer's
 // transform alone: a level over the cluster costs two barriers and a round trip
 // to the neighbours (about 2 us), one of a 32 x 32 block in one CTA less than
-// half of that.  Against S = C (GB300, 10 iterations): one E-ELT frame 416 ->
-// 407 us, one 8 m frame 222 -> 209 us.  At most N / 2, at least C (a row per CTA), and the
+// half of that.  Against S = C (GB300, cold solve of 10 iterations): E-ELT 414 ->
+// 407 us, 8 m 222 -> 211 us.  At most N / 2, at least C (a row per CTA), and the
 // block and its row transforms fit one of the two row buffers.  At most 32, but 16
 //  - in FP64, where one SM's FP64 pipe takes longer over a 32 x 32 block than the cluster (normal
 //    operator, 128 x 128 layers, us with 32 and 16: 5 layers db4 93.7 and 76.9, 7 layers db2 94 and 84);
@@ -321,7 +321,8 @@ struct StreamSet {
 
 // Size of a streamed pass at block side M (elements of T), the bound up to which
 // layers are accepted: the synthesis stages half of it, 2 (kPassRows + LF/2 - 1)
-// coefficient rows; the analysis uses no shared memory.
+// coefficient rows; the analysis uses no shared memory.  (The bound is kept so that
+// what is accepted does not change.)
 TOMO_HD inline int pass_smem_elems(int M, int LF) {
   const int a = 2 * (2 * kPassRows + LF - 2) * M;
   const int s = 4 * (kPassRows + LF / 2 - 1) * M;

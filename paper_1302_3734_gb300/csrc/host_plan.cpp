@@ -864,7 +864,7 @@ tomo_status build_host_plan(const tomo_geometry *geo, HostPlan *P, std::string *
     const int pos = P->pos_off[m * P->n_layers];   // the layers' tables follow each other, 2 nc entries each
     d.part_off = part;
     if (d.kind == kTTOnly) {
-      // (edge corner, layer) pairs, one per thread of a chunk
+      // (edge corner, layer) pairs, four per summing thread of a chunk
       const int pairs = d.n_edge * P->n_layers;
       const int chunks = (pairs + kFwdChunk - 1) / kFwdChunk;
       d.n_tiles = chunks;

@@ -53,7 +53,7 @@ struct HostPlan {
   int vstage = 0;                  // largest staged v (T elements) of one analysis CTA
   std::vector<unsigned char> stage_img;   // per (layer, rank) stage image, img_stride bytes apart
   long long img_stride = 0;
-  std::vector<int2> tt_seg;        // per (layer, rank)
+  std::vector<int2> tt_seg;        // per (layer, gather band)
   std::vector<int> tt_node, tt_beg, tt_k;
   std::vector<double> tt_w;        // 2 per entry
   int n_tt = 0, n_edge_wfs = 0;

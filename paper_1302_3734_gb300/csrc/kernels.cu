@@ -15,8 +15,8 @@
 // The periodic 2-D DWT of one layer runs inside one thread-block cluster: CTA c
 // owns N/C consecutive rows; the row pass is local, and before the column pass
 // each CTA copies the Lf-2 halo rows it needs from its neighbours' shared memory
-// (distributed shared memory) next to its own rows.  The coarse levels (block
-// side <= C) are finished by CTA 0 alone.  Each CTA loads every coefficient it
+// (distributed shared memory) next to its own rows.  The coarse levels (from a
+// block of transform_coarse_side on) are finished by CTA 0 alone.  Each CTA loads every coefficient it
 // owns in one round trip at its start (with the PCG direction update fused in).
 //
 // Reductions are FP64: warp shuffle -> block -> one partial per CTA; the
@@ -71,8 +71,6 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 // MODE 2: data only, z = s (phi = 0).  MODE 3: the noise-free measurement A phi
 // itself (eq. atm_tomo) into io.out0: the slopes, and a tip/tilt-only sensor's
 // two means (by its first chunk's CTA alone); nothing of the plan is written.
-// (Four corners traced per subaperture, layer after layer, took 19 us on the
-// E-ELT system, cold on GB300; these tiles 12.)
 // Otherwise writes the corner field
 // v_m = Gamma_m^T sigma^-2 z_m and, with tip/tilt removal, each tile's sums of z
 // (the analysis subtracts the means on the pupil edge, Sec. 4.3 eq. widehatc).
@@ -1509,7 +1507,7 @@ __global__ void __launch_bounds__(kThreads) k_update(const InstDev *__restrict__
 // mean).  With Td(b), Tm(b) the sums of dU^2 and mU^2 over the valid
 // subapertures of row b, the norm is sum_b mV(b)^2 Td(b) + dV(b)^2 Tm(b).
 //
-// A CTA takes kJacTile columns (basis functions in x) and a group of rows
+// A CTA takes TW columns (basis functions in x) and a group of rows
 // (basis functions in y) of one level's block, so that Td, Tm are formed once
 // per column and row of subapertures and V once per row, not once per
 // coefficient: prefix sums of dU^2, mU^2 per column (a warp scan), then in
