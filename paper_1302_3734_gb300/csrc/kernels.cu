@@ -103,7 +103,8 @@ __device__ __forceinline__ void store_tile_partial(double *slot, Acc<float> a, A
 // of 64 x 64, 9 sensors); 19.7 and 18.7 (7 layers, 7 sensors); 17.7 and 16.8 (8
 // layers of 32 x 32, 6 sensors).
 //
-// Bound by instruction issue and L1 in big launches, by latency in small ones.
+// Bound by the latency of its grid loads (16 E-ELT systems: SM at 45%, L1 at 49% of their
+// peaks; of the reasons a warp waits, the loads are the first).
 // Against one corner per thread on 18 x 18 corners, four loads per corner and
 // layer (GB300, cold launch): 16 E-ELT systems 49.2 -> 29 us, 64 uneven systems
 // 50.9 -> 29 us, the 100 m system 54.0 -> 43 us.

@@ -83,8 +83,8 @@ constexpr int kEmitU = 4;
 // input rows, their row transforms from the lane's window of LF + 2 inputs
 // (16-byte loads; the neighbours' overlap hits the L1), then the column sums
 // over the last LF row transforms, which stay in registers.  No shared memory
-// and no barrier before the partial sums.  Bound by the epilogue's traffic (p in,
-// q out) and the latency of the row loads.  Against staging the tile's rows and
+// and no barrier before the partial sums.  Bound by the latency of the row and
+// epilogue loads (16 E-ELT systems: DRAM at 14%, SM at 25% of their peaks).  Against staging the tile's rows and
 // their row transforms in shared memory for two barrier-separated passes, one
 // output column per thread (GB300, cold launch): finest pass of the 100 m system
 // 51.2 -> 32 us, of 64 uneven systems 71.6 -> 35 us, of 16 E-ELT systems 25.8 ->
@@ -507,8 +507,8 @@ __global__ void __launch_bounds__(kPassThreads) k_idwt_coarse(const InstDev *__r
 // syntheses of the low-y and the high-y row from 16-byte windows, and the column
 // synthesis over the last LF/2 half-rows, whose row syntheses stay in registers.
 // One barrier; a strip repeats the row syntheses of HL half-rows, so a tile has
-// at most four strips.  Bound by the coefficients' loads (DRAM and their latency
-// at four or five CTAs per SM).  Against writing the row syntheses back to shared
+// at most four strips.  Bound by the latency of the coefficients' loads (16
+// E-ELT systems: DRAM at 19%, SM at 24% of their peaks).  Against writing the row syntheses back to shared
 // memory for a second pass (GB300, cold launch): 64 uneven systems 57.7 -> 39 us,
 // 16 E-ELT systems 20.1 -> 14 us, the 100 m system's finest pass 45.4 -> 38 us.
 // (Without the staging, each thread reading its window from global memory, the
